@@ -51,6 +51,11 @@ constexpr double kPi = 3.141592653589793238462643383279502884;
 constexpr int kGraphSteps = 16;  // steps per captured graph (even: buffer parity)
 constexpr int kSlabShift = 4;    // default slab_shift of large runs (rows per step)
 
+// wall-flux partials per wall, whichever step kernel writes them
+int flux_partials(int Nx) {
+  return std::max(march_strips(Nx, 1), std::max(step_flux_blocks(Nx, false), step_flux_blocks(Nx, true)));
+}
+
 size_t storage_bytes(int storage) { return storage == 0 ? 8 : (storage == 1 ? 4 : 2); }
 
 }  // namespace
@@ -266,6 +271,7 @@ StepArgs step_args(const ehd_run* r, int cur) {
   a.wm = 1.0 / r->tau_m;
   a.gwp = 1.0 / r->taug_p;
   a.gwm = 1.0 / r->taug_m;
+  a.k64 = collide_f64_constants(a.wp, a.wm, a.gwp, a.gwm);
   a.mub = r->mub;
   a.rho0 = r->rho0;
   a.wall_mode = r->wall_mode;
@@ -582,7 +588,7 @@ ehd_status ehd_footprint(int Nx, int Ny, int storage, size_t* bytes) {
       ny * 8, ny * rs, ny * Mp * 2 * rs, ny * 8, Mp * ny * rs, ny * 8,         // phibar .. rfac0
       (size_t)(Nx + 1024) * 2 * rs, ny * 4,                                    // twiddles, shifts
       (ny / 4 + 2) * P * rs, (ny / 4 + 2) * P * rs,                            // slab-boundary shares
-      2 * (size_t)std::max(march_strips(Nx, 1), step_flux_blocks(Nx)) * 8,    // flux partials
+      2 * (size_t)flux_partials(Nx) * 8,                                       // flux partials
       16 * 8 + 64, (size_t)reduce_state_blocks() * 6 * 8,
       (3 * (2 * ny + 2) + (size_t)Nx / 2 + 1) * rs,                          // odd-extension tables
       9 * ny * 8, 9 * ny * 8, 9 * ny * 8, 9 * ny * 8, ny * 8, ny * 8, ny * 8,  // perturbation-form base
@@ -760,9 +766,9 @@ ehd_status ehd_create(int Nx, int Ny, double T, double C, double M, double Fe, d
   }
   r->cols_per_lane = 2;
   r->nstrips = march_strips(Nx, r->cols_per_lane);
-  r->nxb = (r->step_kernel == 0) ? r->nstrips : step_flux_blocks(Nx);
+  r->nxb = (r->step_kernel == 0) ? r->nstrips : step_flux_blocks(Nx, r->real_f64);
   r->flux_part = static_cast<double*>(
-      run_alloc(r, 2 * (size_t)std::max(march_strips(Nx, 1), step_flux_blocks(Nx)) * sizeof(double)));
+      run_alloc(r, 2 * (size_t)flux_partials(Nx) * sizeof(double)));
   r->small = static_cast<double*>(run_alloc(r, 16 * sizeof(double) + 64));
   r->red_part = static_cast<double*>(run_alloc(r, (size_t)reduce_state_blocks() * 6 * sizeof(double)));
   bool ok = r->f[0] && r->f[1] && r->g[0] && r->g[1] && r->dphi && r->rhoc && r->rx_dn && r->rx_up && r->phibar &&
@@ -1055,7 +1061,7 @@ ehd_status ehd_tune(ehd_run* r, int param, int value) {
       if (value != 0 && r->pert) return fail(EHD_EINVAL, "perturbation-form runs need the march form");
       if (value != 0 && r->ex_spectral) return fail(EHD_EINVAL, "spectral E_x needs the march form");
       r->step_kernel = value;
-      r->nxb = (value == 0) ? r->nstrips : step_flux_blocks(r->Nx);
+      r->nxb = (value == 0) ? r->nstrips : step_flux_blocks(r->Nx, r->real_f64);
       break;
     default:
       return fail(EHD_EINVAL, "unknown tuning parameter %d", param);

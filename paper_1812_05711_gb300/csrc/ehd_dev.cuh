@@ -111,6 +111,34 @@ cudaError_t tma_encode_2d(CUtensorMap* m, const void* base, unsigned long long i
                           unsigned long long row_bytes, unsigned box_inner, unsigned box_outer);
 cudaError_t modes_tma_encode(ModesTma* t, const void* spec, const void* rfac, int Ny, int Mp);
 
+// Constants of the FP64 collision (collide_f64), formed on the host: an FP64
+// instruction takes its constant operand from the kernel parameters, and no
+// thread spends FP64 issue slots on forming one.
+struct CollideF64 {
+  double hp, hm;        // (1 - omega+) / 2, (1 - omega-) / 2
+  double rw;            // W1 omega+
+  double gj, gF;        // 4.5 W1 omega+, 4.5 W1 (2 - omega+ / 2)
+  double jj, jF;        // 3 W1 omega-, 3 W1
+  double ghp, ghm;      // (1 - omega_g+) / 2, (1 - omega_g-) / 2
+  double grw, gg, gjm;  // W1 omega_g+, 4.5 W1 omega_g+, 3 W1 omega_g-
+};
+inline CollideF64 collide_f64_constants(double wp, double wm, double gwp, double gwm) {
+  CollideF64 k;
+  k.hp = 0.5 * (1.0 - wp);
+  k.hm = 0.5 * (1.0 - wm);
+  k.rw = kW1 * wp;
+  k.gj = 4.5 * kW1 * wp;
+  k.gF = 4.5 * kW1 * (2.0 - 0.5 * wp);
+  k.jj = 3.0 * kW1 * wm;
+  k.jF = 3.0 * kW1;
+  k.ghp = 0.5 * (1.0 - gwp);
+  k.ghm = 0.5 * (1.0 - gwm);
+  k.grw = kW1 * gwp;
+  k.gg = 4.5 * kW1 * gwp;
+  k.gjm = 3.0 * kW1 * gwm;
+  return k;
+}
+
 struct StepArgs {
   int Nx, Ny, P;
   long long plane;           // elements per population plane (Ny * P)
@@ -140,7 +168,98 @@ struct StepArgs {
   int cols_per_lane;         // 1: 32-column strips (30 owned); 2: 64-column strips (60 owned)
   int pdl;                   // launch with programmatic dependent launch (see launch_ex)
   const float* base_tab;     // perturbation form: the march table of time t ([Ny][4]); nullptr otherwise
+  CollideF64 k64;            // constants of the FP64 collision
 };
+
+// -------------------------------------------------- FP64 TRT collision ---
+// Scalar FP64 issues two lanes per clock and SM on this part (a warp's FP64
+// instruction takes the unit 16 cycles), so the FP64 step is bound by its FP64
+// instruction count and nothing else.  This is the collision of Eqs. 5-15
+// with that count at about 130 per node (226 when every population's
+// equilibrium, force and relaxation were formed one by one as in the FP32
+// kernels):
+//   - sums s and differences d of each pair of opposite populations serve the
+//     moments and the relaxation alike;
+//   - the post-collision pair is P + D, P - D with P = (1 - omega+) s / 2 +
+//     E, D = (1 - omega-) d / 2 + J; since rho u = j + F / 2 (Eq. 7), the
+//     equilibrium and the force enter E and J only through
+//     G = 4.5 W1 (omega+ j + (2 - omega+ / 2) F) and 3 W1 (omega- j + F):
+//     with C = W1 omega+ rho - u.G / 3 the axis pairs get C + u_x G_x and
+//     C + u_y G_y, and the diagonal pairs a quarter of
+//     C + u.G +- (u_x G_y + u_y G_x);
+//   - the rest population takes what the pairs leave of the density, so the
+//     mass and charge of a node are conserved to a rounding that has no
+//     preferred sign, whatever the rounding of the constants;
+//   - 1 / rho by one third-order Householder step x (1 + e + e^2), e = 1 -
+//     rho x, from the hardware's approximation.
+__device__ __forceinline__ double recip_f64(double v) {
+  double x;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(v));
+  const double e = fma(-v, x, 1.0);
+  return fma(x, fma(e, e, e), x);
+}
+// finite: the exponent bits are not all ones (an integer test: an FP64
+// compare would take an FP64 slot)
+__device__ __forceinline__ bool finite_f64(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
+__device__ __forceinline__ void collide_f64(double (&f)[9], double (&g)[9], double Ex, double Ey, double mub,
+                                            const CollideF64& k, bool& bad) {
+  constexpr double third = -1.0 / 3.0;
+  // fluid
+  const double s1 = f[1] + f[3], s2 = f[2] + f[4], s5 = f[5] + f[7], s6 = f[6] + f[8];
+  const double d1 = f[1] - f[3], d2 = f[2] - f[4], d5 = f[5] - f[7], d6 = f[6] - f[8];
+  const double rho = ((s1 + s2) + (s5 + s6)) + f[0];
+  const double jx = d1 + (d5 - d6), jy = d2 + (d5 + d6);
+  // charge
+  const double p1 = g[1] + g[3], p2 = g[2] + g[4], p5 = g[5] + g[7], p6 = g[6] + g[8];
+  const double e1 = g[1] - g[3], e2 = g[2] - g[4], e5 = g[5] - g[7], e6 = g[6] - g[8];
+  const double rc = ((p1 + p2) + (p5 + p6)) + g[0];
+  bad = !finite_f64(rho) || !finite_f64(rc);
+  const double Fx = rc * Ex, Fy = rc * Ey;
+  const double irho = recip_f64(rho);
+  const double ux = fma(0.5, Fx, jx) * irho, uy = fma(0.5, Fy, jy) * irho;
+  {
+    const double Gx = fma(k.gj, jx, k.gF * Fx), Gy = fma(k.gj, jy, k.gF * Fy);
+    const double Q = fma(uy, Gy, ux * Gx), X = fma(ux, Gy, uy * Gx);
+    const double C = fma(third, Q, k.rw * rho), t = 0.25 * (C + Q);
+    const double P1 = fma(k.hp, s1, fma(ux, Gx, C)), P2 = fma(k.hp, s2, fma(uy, Gy, C));
+    const double P5 = fma(k.hp, s5, fma(0.25, X, t)), P6 = fma(k.hp, s6, fma(-0.25, X, t));
+    const double Jx = fma(k.jj, jx, k.jF * Fx), Jy = fma(k.jj, jy, k.jF * Fy);
+    const double D1 = fma(k.hm, d1, Jx), D2 = fma(k.hm, d2, Jy);
+    const double q = 0.25 * Jy;
+    const double D5 = fma(k.hm, d5, fma(0.25, Jx, q)), D6 = fma(k.hm, d6, fma(-0.25, Jx, q));
+    f[0] = fma(-2.0, (P1 + P2) + (P5 + P6), rho);
+    f[1] = P1 + D1;
+    f[3] = P1 - D1;
+    f[2] = P2 + D2;
+    f[4] = P2 - D2;
+    f[5] = P5 + D5;
+    f[7] = P5 - D5;
+    f[6] = P6 + D6;
+    f[8] = P6 - D6;
+  }
+  {
+    const double vx = fma(mub, Ex, ux), vy = fma(mub, Ey, uy);
+    const double h = k.gg * rc, Gx = h * vx, Gy = h * vy, X = vx * Gy;  // v_x G_y = v_y G_x
+    const double Q = fma(vy, Gy, vx * Gx);
+    const double C = fma(third, Q, k.grw * rc), t = 0.25 * (C + Q);
+    const double P1 = fma(k.ghp, p1, fma(vx, Gx, C)), P2 = fma(k.ghp, p2, fma(vy, Gy, C));
+    const double P5 = fma(k.ghp, p5, fma(0.5, X, t)), P6 = fma(k.ghp, p6, fma(-0.5, X, t));
+    const double m = k.gjm * rc, Jx = m * vx, Jy = m * vy;
+    const double D1 = fma(k.ghm, e1, Jx), D2 = fma(k.ghm, e2, Jy);
+    const double q = 0.25 * Jy;
+    const double D5 = fma(k.ghm, e5, fma(0.25, Jx, q)), D6 = fma(k.ghm, e6, fma(-0.25, Jx, q));
+    g[0] = fma(-2.0, (P1 + P2) + (P5 + P6), rc);
+    g[1] = P1 + D1;
+    g[3] = P1 - D1;
+    g[2] = P2 + D2;
+    g[4] = P2 - D2;
+    g[5] = P5 + D5;
+    g[7] = P5 - D5;
+    g[6] = P6 + D6;
+    g[8] = P6 - D6;
+  }
+}
 
 struct PoissonArgs {
   int Nx, Ny, P, Mh, log2Nx;
@@ -353,7 +472,7 @@ cudaError_t launch_march_tma(const StepArgs& a, const MarchTma& m, int form, cud
 // Launchers (defined in the .cu files); storage: 0 F64, 1 F32, 2 BF16, 3 F16;
 // real_f64: compute type (true = double).
 cudaError_t launch_step(const StepArgs& a, int storage, bool real_f64, int rows_per_cta, cudaStream_t s);
-int step_flux_blocks(int Nx);
+int step_flux_blocks(int Nx, bool real_f64);
 cudaError_t launch_march(const StepArgs& a, int storage, bool real_f64, cudaStream_t s);
 int march_strips(int Nx, int cols_per_lane);
 int march_warps_per_sm(int storage, bool real_f64, int cols_per_lane, int ring_depth);

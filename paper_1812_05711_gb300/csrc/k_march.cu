@@ -467,7 +467,11 @@ struct March2Stages {
 
 template <class S, class R>
 __device__ __forceinline__ void collide_node(R (&f)[9], R (&g)[9], R Ex, R Ey, R sy, R sf, R dq, R mub, R wp, R wm,
-                                             R cp, R cm, R gwp, R gwm, bool& bad) {
+                                             R cp, R cm, R gwp, R gwm, const CollideF64& k64, bool& bad) {
+  if constexpr (sizeof(R) == 8) {  // unshifted: sy, sf and dq are zero
+    collide_f64(f, g, Ex, Ey, mub, k64, bad);
+    return;
+  }
   const R W0 = (R)kW0, W1 = (R)kW1, W2 = (R)kW2;
   const R drho = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
   const R rho = sf + drho;
@@ -723,8 +727,8 @@ __device__ __forceinline__ void march2_body(const StepArgs& a, int strip, int sl
       collide_node_pert<R>(f0, g0, Ex0, EB + Ey0, Ey0, sy, uBy, vby, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, b0);
       collide_node_pert<R>(f1, g1, Ex1, EB + Ey1, Ey1, sy, uBy, vby, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, b1);
     } else {
-      collide_node<S, R>(f0, g0, Ex0, Ey0, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, b0);
-      collide_node<S, R>(f1, g1, Ex1, Ey1, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, b1);
+      collide_node<S, R>(f0, g0, Ex0, Ey0, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, a.k64, b0);
+      collide_node<S, R>(f1, g1, Ex1, Ey1, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, a.k64, b1);
     }
     if (owned && (b0 || b1)) bad = true;
     // pulled values at (xc, xc + 1): x-shift by c_x
@@ -1273,8 +1277,8 @@ __device__ __forceinline__ void march_tma_body(const StepArgs& a, const MarchTma
       g1[i] = G[i][1];
     }
     bool b0, b1;
-    collide_node<float, R>(f0, g0, Ex0, Ey0, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, b0);
-    collide_node<float, R>(f1, g1, Ex1, Ey1, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, b1);
+    collide_node<float, R>(f0, g0, Ex0, Ey0, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, a.k64, b0);
+    collide_node<float, R>(f1, g1, Ex1, Ey1, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, a.k64, b1);
     if (owned && (b0 || b1)) bad = true;
     const R P1f0 = from_left(f1[1]), P5f0 = from_left(f1[5]), P8f0 = from_left(f1[8]);
     const R P3f1 = from_right(f0[3]), P6f1 = from_right(f0[6]), P7f1 = from_right(f0[7]);

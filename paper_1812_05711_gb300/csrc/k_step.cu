@@ -214,7 +214,117 @@ __global__ void __launch_bounds__(kStepThreads) k_step(StepArgs a, int rows) {
   }
 }
 
-int step_flux_blocks(int Nx) { return (Nx + kStepThreads - 1) / kStepThreads; }
+// The FP64 form: one warp per 32 nodes of a row.  Bound by its FP64
+// instructions (collide_f64), so what counts beside their number is an even
+// share for every SM: one-warp CTAs leave at most one warp's difference
+// between SMs (128 x 104: three warps on the fullest SM, four with two-warp
+// CTAs and eight with four; the loads of up to 16 resident warps overlap the
+// arithmetic).  FP64 storage is unshifted (rch == nullptr, fb = fd = 0).
+constexpr int kStep64Threads = 32;
+__global__ void __launch_bounds__(kStep64Threads, 16) k_step64(StepArgs a) {
+  const int x = blockIdx.x * kStep64Threads + threadIdx.x, y = blockIdx.y;
+  const int Nx = a.Nx, Ny = a.Ny, P = a.P;
+  const long long pl = a.plane;
+  double* __restrict__ fo = static_cast<double*>(a.fout);
+  double* __restrict__ go = static_cast<double*>(a.gout);
+  double qin = 0.0, qout = 0.0;
+  const bool live = x < Nx;
+  double f[9], g[9];
+  const long long c = (long long)y * P + x;
+  if (live) {
+    // the populations were written by the previous step's launch of this
+    // kernel: loaded before the wait for the potential (see grid_dep_wait)
+    const double* __restrict__ fin = static_cast<const double*>(a.fin) + c;
+    const double* __restrict__ gin = static_cast<const double*>(a.gin) + c;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      f[i] = __ldg(fin + i * pl);
+      g[i] = __ldg(gin + i * pl);
+    }
+  }
+  grid_dep_wait();
+  if (live) {
+    const int xl = (x == 0) ? Nx - 1 : x - 1;
+    const int xr = (x == Nx - 1) ? 0 : x + 1;
+    // E = -grad phi, central differences; phi = phibar(y) + dphi
+    const double* __restrict__ dp = static_cast<const double*>(a.dphi) + c;
+    const double gwall = (a.wall_mode == 0) ? -1.0 : 0.0;
+    const double pW = __ldg(dp - x + xl), pE = __ldg(dp - x + xr);
+    const double pS = (y > 0) ? __ldg(dp - P) : gwall * __ldg(dp);
+    const double pN = (y < Ny - 1) ? __ldg(dp + P) : gwall * __ldg(dp);
+    const double Ex = -0.5 * (pE - pW);
+    const double Ey = fma(-0.5, pN - pS, __ldg(static_cast<const double*>(a.Ebar) + y));
+    bool bad;
+    collide_f64(f, g, Ex, Ey, a.mub, a.k64, bad);
+    if (bad) atomicOr(a.err, 1);
+    // streaming: f_i(x + c_i, t + 1) = f_i*(x, t)
+    const long long yo = (long long)y * P;
+    fo[yo + x] = f[0];
+    go[yo + x] = g[0];
+    fo[pl + yo + xr] = f[1];
+    go[pl + yo + xr] = g[1];
+    fo[3 * pl + yo + xl] = f[3];
+    go[3 * pl + yo + xl] = g[3];
+    if (y + 1 < Ny) {
+      const long long yu = yo + P;
+      fo[2 * pl + yu + x] = f[2];
+      go[2 * pl + yu + x] = g[2];
+      fo[5 * pl + yu + xr] = f[5];
+      go[5 * pl + yu + xr] = g[5];
+      fo[6 * pl + yu + xl] = f[6];
+      go[6 * pl + yu + xl] = g[6];
+    } else {
+      // collector: f bounces back into its own node, g leaves the channel and
+      // the downward populations entering from the wall side are the node's
+      // own post-collision values (zero-gradient outflow)
+      fo[4 * pl + yo + x] = f[2];
+      fo[7 * pl + yo + x] = f[5];
+      fo[8 * pl + yo + x] = f[6];
+      go[4 * pl + yo + x] = g[4];
+      go[7 * pl + yo + xl] = g[7];
+      go[8 * pl + yo + xr] = g[8];
+      qout = ((g[2] + g[5]) + g[6]) - ((g[4] + g[7]) + g[8]);
+    }
+    if (y > 0) {
+      const long long yd = yo - P;
+      fo[4 * pl + yd + x] = f[4];
+      go[4 * pl + yd + x] = g[4];
+      fo[7 * pl + yd + xl] = f[7];
+      go[7 * pl + yd + xl] = g[7];
+      fo[8 * pl + yd + xr] = f[8];
+      go[8 * pl + yd + xr] = g[8];
+    } else {
+      // injector: halfway bounce-back of f; anti-bounce-back of g imposing
+      // rho_c = rho0 with the wall drift mu_b E (fluid at rest on the wall)
+      fo[2 * pl + yo + x] = f[4];
+      fo[5 * pl + yo + x] = f[7];
+      fo[6 * pl + yo + x] = f[8];
+      const double wx = a.mub * Ex, wy = a.mub * Ey;
+      const double w15 = 1.5 * (wx * wx + wy * wy);
+      const double c2 = wy, c5 = wx + wy, c6 = wy - wx;
+      const double n2 = -g[4] + 2.0 * kW1 * a.rho0 * (1.0 + 4.5 * c2 * c2 - w15);
+      const double n5 = -g[7] + 2.0 * kW2 * a.rho0 * (1.0 + 4.5 * c5 * c5 - w15);
+      const double n6 = -g[8] + 2.0 * kW2 * a.rho0 * (1.0 + 4.5 * c6 * c6 - w15);
+      go[2 * pl + yo + x] = n2;
+      go[5 * pl + yo + x] = n5;
+      go[6 * pl + yo + x] = n6;
+      qin = ((n2 - g[4]) + (n5 - g[7])) + (n6 - g[8]);
+    }
+  }
+  if (y == 0) {
+    for (int o = 16; o > 0; o >>= 1) qin += __shfl_down_sync(0xffffffffu, qin, o);
+    if (threadIdx.x == 0) a.flux_part[blockIdx.x] = qin;
+  }
+  if (y == Ny - 1) {
+    for (int o = 16; o > 0; o >>= 1) qout += __shfl_down_sync(0xffffffffu, qout, o);
+    if (threadIdx.x == 0) a.flux_part[gridDim.x + blockIdx.x] = qout;
+  }
+}
+
+int step_flux_blocks(int Nx, bool real_f64) {
+  const int n = real_f64 ? kStep64Threads : kStepThreads;
+  return (Nx + n - 1) / n;
+}
 
 namespace {
 template <class S, class R>
@@ -228,7 +338,8 @@ cudaError_t step_t(const StepArgs& a, int rows, cudaStream_t s) {
 cudaError_t launch_step(const StepArgs& a, int storage, bool real_f64, int rows, cudaStream_t s) {
   if (real_f64) {
     if (storage != 0) return cudaErrorInvalidValue;
-    return step_t<double, double>(a, rows, s);
+    return launch_ex((a.pdl & 8) != 0, k_step64, dim3((a.Nx + kStep64Threads - 1) / kStep64Threads, a.Ny),
+                     dim3(kStep64Threads), 0, s, a);
   }
   switch (storage) {
     case 0: return step_t<double, float>(a, rows, s);
