@@ -410,14 +410,21 @@ cudaError_t enqueue_base(ehd_run* r, int cur) {
 // Charge plane of buffer `cur`, then phi (the Poisson solve).  Perturbation
 // form: the departure's charge and potential, and the base's potential.
 cudaError_t enqueue_poisson(ehd_run* r, int cur, bool with_flux) {
-  cudaError_t e = launch_rhoc(r->g[cur], (long long)r->Ny * r->P, r->storage, r->real_f64, r->Nx, r->Ny, r->P,
-                              r->pert ? nullptr : r->rch, r->rhoc, r->stream);
-  if (e != cudaSuccess) return e;
+  PoissonArgs pa = poisson_args(r, with_flux);
+  cudaError_t e = cudaSuccess;
+  if (r->real_f64) {  // the forward transform sums the populations
+    pa.g = r->g[cur];
+    pa.gplane = (long long)r->Ny * r->P;
+  } else {
+    e = launch_rhoc(r->g[cur], (long long)r->Ny * r->P, r->storage, r->Nx, r->Ny, r->P, r->pert ? nullptr : r->rch,
+                    r->rhoc, r->stream);
+    if (e != cudaSuccess) return e;
+  }
   if (r->pert) {
     if ((e = launch_base_sums(base_step_args(r, cur), r->stream)) != cudaSuccess) return e;
     if ((e = launch_base_poisson(base_poisson_args(r, cur), r->stream)) != cudaSuccess) return e;
   }
-  return launch_poisson(poisson_args(r, with_flux), r->real_f64, r->stream, r->side, r->ev_fork, r->ev_join);
+  return launch_poisson(pa, r->real_f64, r->stream, r->side, r->ev_fork, r->ev_join);
 }
 
 FieldArgs field_args(const ehd_run* r) {
@@ -762,7 +769,10 @@ ehd_status ehd_create(int Nx, int Ny, double T, double C, double M, double Fe, d
   // transform CTAs starve the base chain on the third stream)
   {
     const long long nodes = (long long)Nx * Ny;
-    r->pdl = (r->pert || (nodes > (1LL << 18) && nodes < (1LL << 21))) ? 11 : 7;
+    // FP64 runs: every kernel; none of them releases its successor early (see
+    // k_modes64), so that all sizes gain or break even (16 x 100: 22.4 us
+    // against 23.2 without; 128 x 104: 25.1 / 25.3; 1024 x 840: 317.3 / 317.3)
+    r->pdl = r->real_f64 ? 15 : (r->pert || (nodes > (1LL << 18) && nodes < (1LL << 21))) ? 11 : 7;
   }
   r->cols_per_lane = 2;
   r->nstrips = march_strips(Nx, r->cols_per_lane);
@@ -1149,9 +1159,12 @@ ehd_status ehd_step_profile(ehd_run* r, long n, double* ms_out) {
       e = (r->step_kernel == 0) ? launch_march_run(r, sa, r->cur)
                                 : launch_step(sa, r->storage, r->real_f64, r->rows, r->stream);
     if (e == cudaSuccess) e = cudaEventRecord(E[1], r->stream);
-    if (e == cudaSuccess && r->step_kernel == 1)
-      e = launch_rhoc(r->g[nxt], (long long)r->Ny * r->P, r->storage, r->real_f64, r->Nx, r->Ny, r->P, r->rch,
-                      r->rhoc, r->stream);
+    if (r->real_f64 && r->step_kernel == 1) {
+      pa.g = r->g[nxt];
+      pa.gplane = (long long)r->Ny * r->P;
+    } else if (e == cudaSuccess && r->step_kernel == 1) {
+      e = launch_rhoc(r->g[nxt], (long long)r->Ny * r->P, r->storage, r->Nx, r->Ny, r->P, r->rch, r->rhoc, r->stream);
+    }
     if (e == cudaSuccess) e = cudaEventRecord(E[2], r->stream);
     if (e == cudaSuccess)
       e = launch_poisson(pa, r->real_f64, r->stream, r->side, r->ev_fork, r->ev_join, E + 4);

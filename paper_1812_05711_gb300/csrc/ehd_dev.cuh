@@ -265,6 +265,8 @@ struct PoissonArgs {
   int Nx, Ny, P, Mh, log2Nx;
   int Mp;                    // row pitch of the spectrum and pivot tables (Mh rounded up to 4)
   const void* rhoc;          // charge density, R [Ny][P]
+  const void* g;             // FP64: charge populations whose sum is the charge density (rhoc then unused), or nullptr
+  long long gplane;          // elements per plane of g
   const void* rhoc_dn;       // slab-boundary partials of the march form (see StepArgs), added to rhoc
   const void* rhoc_up;
   int xslab;                 // slab height of those partials; 0: rhoc is complete
@@ -482,6 +484,9 @@ cudaError_t march_set_attributes();
 // between the fork and join events when side != nullptr.
 cudaError_t launch_poisson(const PoissonArgs& a, bool real_f64, cudaStream_t s, cudaStream_t side, cudaEvent_t fork,
                            cudaEvent_t join, const cudaEvent_t* marks = nullptr);
+// row transforms of the FP64 path (k_fft64.cu); the spectrum they keep is S / Nx
+cudaError_t launch_rfft64(const PoissonArgs& a, cudaStream_t s);
+cudaError_t launch_irfft64(const PoissonArgs& a, bool dx, cudaStream_t s);
 // Odd-extension y solve (k_oddext.cu): radices of n (4, 2, 3, 5, 7, 11, 13;
 // at most cap of them) into fac, their count, or -1 if n has another factor;
 // the shared memory one CTA needs; the launch over m = 1 .. Mh - 1.
@@ -489,8 +494,8 @@ int oddext_factors(int n, int* fac, int cap);
 size_t oddext_smem_bytes(int NE, bool real_f64);
 cudaError_t launch_modes_oddext(const PoissonArgs& a, bool real_f64, cudaStream_t s);
 cudaError_t oddext_set_attributes();
-// rho_c = sum_i g_i (+ the row shift) into the charge plane.
-cudaError_t launch_rhoc(const void* g, long long plane, int storage, bool real_f64, int Nx, int Ny, int P,
+// rho_c = sum_i g_i (+ the row shift) into the charge plane (FP32 compute).
+cudaError_t launch_rhoc(const void* g, long long plane, int storage, int Nx, int Ny, int P,
                         const float* rch, void* rhoc, cudaStream_t s);
 cudaError_t poisson_set_attributes();
 // warp-per-row real FFTs (FP32 path, Nx = 64 ... 2048)

@@ -7,18 +7,21 @@
 //
 //   k_rhoc        rho_c = sum_i g_i (Eq. 6) from the populations, when the
 //                 step kernel did not already write it.
-//   k_rfft_rows   1024/L rows per CTA (L = Nx/2): the row's N real samples are
-//                 packed as L complex values, transformed by a radix-4
-//                 Stockham FFT in shared memory and untangled into the half
-//                 spectrum (Eq. 19).  The row mean (the m = 0 mode) is summed
-//                 in FP32 pairs with a compensated tree and removed first.
+//   k_rfft_rows   FP32 rows of 16 and 32 (wider ones: k_fftw.cu; FP64:
+//                 k_fft64.cu), 1024/L rows per CTA (L = Nx/2): the row's N
+//                 real samples are packed as L complex values, transformed
+//                 by a radix-4 Stockham FFT in shared memory and untangled
+//                 into the half spectrum (Eq. 19).  The row mean (the m = 0
+//                 mode) is summed in FP32 pairs with a compensated tree and
+//                 removed first.
 //   k_modes_tile  8 wavenumbers x Ny rows per CTA held in shared memory; the
 //                 Thomas recurrences of each wavenumber (reciprocal pivots
 //                 precomputed) run as 32 chunk-parallel affine scans.
-//   k_mean_mode   128 threads: the m = 0 system in FP64 with the wall
-//                 potentials lifted into the right-hand side; also adds the
-//                 step's wall-flux partials to the run's FP64 totals.  It
-//                 runs on a second stream, beside k_modes_tile/k_rfft_inv.
+//   k_mean_mode   128 threads: the m = 0 system with the wall potentials
+//                 lifted into the right-hand side; also adds the step's
+//                 wall-flux partials to the run's FP64 totals.  It runs on a
+//                 second stream, beside k_modes_tile / the inverse.
+//   k_modes64     both of these for the FP64 path, one warp per wavenumber.
 //   k_irfft_rows  inverse of k_rfft_rows -> phi minus its row mean.
 #include <algorithm>
 
@@ -150,11 +153,10 @@ __global__ void k_rhoc(const S* __restrict__ g, long long plane, int Nx, int Ny,
 
 // ------------------------------------------------------------ forward FFT ---
 // Shared memory: twiddle table (N complex), then per row two padded buffers.
-template <class R>
 __global__ void __launch_bounds__(256) k_rfft_rows(PoissonArgs a) {
+  using R = float;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ float wred_hi[8], wred_lo[8];
-  __shared__ double wred_d[8];
   const int N = a.Nx, L = N >> 1;
   const int T = (L >= 4) ? (L >> 2) : 1;  // threads per row
   const int rows = 256 / T;
@@ -195,19 +197,8 @@ __global__ void __launch_bounds__(256) k_rfft_rows(PoissonArgs a) {
   // within segments of min(T, 32) lanes, then the row's warps
   const int W = T < 32 ? T : 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float shi = 0.0f, slo = 0.0f;  // FP32 path: float-float
-  double sd = 0.0;               // FP64 path
-  if constexpr (sizeof(R) == 8) {
-    sd = (double)part;
-    for (int o = W >> 1; o > 0; o >>= 1) sd += __shfl_down_sync(0xffffffffu, sd, o, W);
-    if (T > 32) {
-      if (lane == 0) wred_d[warp] = sd;
-      __syncthreads();
-      if (tr == 0)
-        for (int w = 1; w < T / 32; ++w) sd += wred_d[warp + w];
-    }
-  } else {
-    shi = (float)part;
+  float shi = (float)part, slo = 0.0f;  // float-float
+  {
     for (int o = W >> 1; o > 0; o >>= 1) {
       const float h2 = __shfl_down_sync(0xffffffffu, shi, o, W), l2 = __shfl_down_sync(0xffffffffu, slo, o, W);
       float s_, e_;
@@ -232,15 +223,10 @@ __global__ void __launch_bounds__(256) k_rfft_rows(PoissonArgs a) {
   }
   __shared__ R rmean[256 / 2];  // rows per CTA <= 128
   if (tr == 0) {
-    if constexpr (sizeof(R) == 8) {
-      if (live) static_cast<double*>(a.spec0)[y] = sd;
-      rmean[lr] = (R)(sd / (double)N);
-    } else {
-      float h, l;  // renormalise
-      two_sum(shi, slo, h, l);
-      if (live) static_cast<float2*>(a.spec0)[y] = make_float2(h, l);
-      rmean[lr] = h / (float)N;
-    }
+    float h, l;  // renormalise
+    two_sum(shi, slo, h, l);
+    if (live) static_cast<float2*>(a.spec0)[y] = make_float2(h, l);
+    rmean[lr] = h / (float)N;
   }
   __syncthreads();
   const R mean = rmean[lr];
@@ -282,8 +268,9 @@ __device__ __forceinline__ Cplx<R> spec_coef(const Cplx<R>* spec, int k, int L) 
   }
 }
 
-template <class R, bool DX = false>
+template <bool DX = false>
 __global__ void __launch_bounds__(256) k_irfft_rows(PoissonArgs a) {
+  using R = float;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int N = a.Nx, L = N >> 1;
   const int T = (L >= 4) ? (L >> 2) : 1;
@@ -320,10 +307,7 @@ __global__ void __launch_bounds__(256) k_irfft_rows(PoissonArgs a) {
     const R inL = R(1) / (R)L;
     for (int n = tr; n < L; n += T) {
       const Cplx<R> v = zr[pidx(n)];
-      if constexpr (sizeof(R) == 4)
-        reinterpret_cast<float2*>(dphi)[n] = make_float2(v.re * inL, v.im * inL);
-      else
-        reinterpret_cast<double2*>(dphi)[n] = make_double2(v.re * inL, v.im * inL);
+      reinterpret_cast<float2*>(dphi)[n] = make_float2(v.re * inL, v.im * inL);
     }
   }
 }
@@ -335,6 +319,13 @@ __global__ void __launch_bounds__(256) k_irfft_rows(PoissonArgs a) {
 // A CTA holds MB wavenumbers x Ny rows in shared memory; thread (chunk, mode)
 // composes the affine maps of its chunk of rows, the chunk maps are combined
 // in order, then each chunk is evaluated from its carried-in value.
+// Barrier among the first NT threads of the CTA that solve a tile (the CTA
+// may have more; see k_modes64).
+template <int NT>
+__device__ __forceinline__ void tile_sync() {
+  asm volatile("bar.sync 2, %0;\n" ::"n"(NT) : "memory");
+}
+
 template <class R, int MB, int NT>
 struct TileScratch {
   R al[NT / MB][MB];
@@ -379,7 +370,7 @@ __device__ __forceinline__ void chunk_carries(TileScratch<R, MB, NT>& ts) {
       ts.wa[mo][seg] = al;
       ts.wb[mo][seg] = br;
     }
-    __syncthreads();
+    tile_sync<NT>();
     for (int k = 0; k < seg; ++k) {
       const R ak = ts.wa[mo][k];
       const Cplx<R> bk = ts.wb[mo][k];
@@ -422,7 +413,7 @@ __device__ __forceinline__ void modes_tile_body(const PoissonArgs& a, int m0, un
     }
     if constexpr (PDL) {
       grid_dep_wait();
-      grid_dep_launch();
+      if constexpr (sizeof(R) == 4) grid_dep_launch();
     }
     for (int idx = threadIdx.x; idx < Ny * CPR; idx += NT) {
       const int j = idx / CPR, c = idx % CPR;
@@ -431,7 +422,7 @@ __device__ __forceinline__ void modes_tile_body(const PoissonArgs& a, int m0, un
     }
     cp_async_all();
   }
-  __syncthreads();
+  tile_sync<NT>();
   modes_tile_sweeps<R, MB, NT>(a, m0, d, rt, ts);
 }
 
@@ -456,13 +447,22 @@ __device__ __forceinline__ void modes_tile_sweeps(const PoissonArgs& a, int m0, 
     const R r = rt[j * MB + mo];
     const Cplx<R> dj = d[j * MB + mo];
     al = -r * al;
-    br = {r * (dj.re - br.re), r * (dj.im - br.im)};
+    if constexpr (sizeof(R) == 8) {
+      // FP64 issue is what bounds these sweeps: r d is formed once and kept,
+      // each sweep is then one fused multiply-add per part (12 FP64
+      // instructions per value instead of 14)
+      const Cplx<R> rd = {r * dj.re, r * dj.im};
+      d[j * MB + mo] = rd;
+      br = {fma(-r, br.re, rd.re), fma(-r, br.im, rd.im)};
+    } else {
+      br = {r * (dj.re - br.re), r * (dj.im - br.im)};
+    }
   }
   s_al[ch][mo] = al;
   s_br[ch][mo] = br;
-  __syncthreads();
+  tile_sync<NT>();
   chunk_carries<R, MB, NT, false>(ts);  // value entering each chunk
-  __syncthreads();
+  tile_sync<NT>();
   // forward evaluation; compose the backward chunk map on the way
   Cplx<R> x = s_carry[ch][mo];
   R ab = R(1);
@@ -470,17 +470,20 @@ __device__ __forceinline__ void modes_tile_sweeps(const PoissonArgs& a, int m0, 
   for (int j = j0; j < j1; ++j) {
     const R r = rt[j * MB + mo];
     const Cplx<R> dj = d[j * MB + mo];
-    x = {r * (dj.re - x.re), r * (dj.im - x.im)};
+    if constexpr (sizeof(R) == 8)
+      x = {fma(-r, x.re, dj.re), fma(-r, x.im, dj.im)};
+    else
+      x = {r * (dj.re - x.re), r * (dj.im - x.im)};
     d[j * MB + mo] = x;
     bb = {bb.re + ab * x.re, bb.im + ab * x.im};
     ab = -ab * r;
   }
-  __syncthreads();
+  tile_sync<NT>();
   s_al[ch][mo] = ab;
   s_br[ch][mo] = bb;
-  __syncthreads();
+  tile_sync<NT>();
   chunk_carries<R, MB, NT, true>(ts);  // value just above each chunk, from the top down
-  __syncthreads();
+  tile_sync<NT>();
   // backward evaluation, each solved value stored as it is formed (a warp's
   // store covers 8 wavenumbers of 4 rows, 64 contiguous bytes each); the
   // stores issue while the sweep's dependent chain waits
@@ -961,6 +964,32 @@ __global__ void __launch_bounds__(NT) k_mean_mode(PoissonArgs a) {
   mean_mode_body<R, NT>(a, smem_raw, ms);
 }
 
+// The FP64 y solve of one run in one launch: CTA 0 the mean mode, the others
+// MB wavenumbers each, one warp per wavenumber.  In a launch of its own on a
+// second stream the mean mode cost a step the fork and the join.  No early
+// release of the inverse transform: its CTAs, resident early, would share
+// SMs unevenly with these (a warp's FP64 instruction takes 64 cycles of its
+// scheduler's quarter of the SM).
+constexpr int kMeanThreads64 = 128;
+constexpr int modes64_threads(int MB) { return 32 * MB > kMeanThreads64 ? 32 * MB : kMeanThreads64; }
+template <int MB>
+__global__ void __launch_bounds__(modes64_threads(MB)) k_modes64(PoissonArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ union Scratch {
+    __device__ Scratch() {}
+    TileScratch<double, MB, 32 * MB> ts;
+    MeanScratch<double, kMeanThreads64> ms;
+  } sc;
+  if (blockIdx.x == 0) {
+    if (threadIdx.x >= kMeanThreads64) return;
+    grid_dep_wait();
+    mean_mode_body<double, kMeanThreads64>(a, smem_raw, sc.ms);
+  } else {
+    if (threadIdx.x >= 32 * MB) return;
+    modes_tile_body<double, MB, 32 * MB, true>(a, (blockIdx.x - 1) * MB, smem_raw, sc.ts);
+  }
+}
+
 // Batch kernels: CTAs take (run, tile) items / one CTA per run.
 __global__ void __launch_bounds__(kTileThreads) k_batch_modes(BatchTables t, int step) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1437,14 +1466,34 @@ int tile_modes(int Ny, size_t cbytes, size_t rbytes) {
   return mb;
 }
 
-template <class R>
+// The FP64 y solve: one warp per wavenumber -- the solves are bound by FP64
+// issue, so they are spread over as many SMs as there are wavenumbers, and
+// from there on in pairs (whole 32-byte sectors of the spectrum's rows) --
+// and the mean mode in a CTA of the same launch.
+template <int MB>
+cudaError_t modes64_n(const PoissonArgs& a, cudaStream_t s) {
+  const size_t tile = (size_t)a.Ny * MB * 3 * sizeof(double), mean = 2 * (size_t)a.Ny * sizeof(double);
+  return launch_ex((a.pdl & 2) != 0, k_modes64<MB>, dim3(1 + (a.Mh + MB - 1) / MB), dim3(modes64_threads(MB)),
+                   std::max(tile, mean), s, a);
+}
+cudaError_t launch_modes64(const PoissonArgs& a, cudaStream_t s) {
+  const int fit = tile_modes(a.Ny, sizeof(Cplx<double>), sizeof(double));
+  switch (std::min(fit, a.tile_modes > 0 ? a.tile_modes : (a.Mh > 152 ? 2 : 1))) {
+    case 8: return modes64_n<8>(a, s);
+    case 4: return modes64_n<4>(a, s);
+    case 2: return modes64_n<2>(a, s);
+    default: return modes64_n<1>(a, s);
+  }
+}
+
 cudaError_t launch_modes(const PoissonArgs& a, cudaStream_t s) {
+  using R = float;
   int mb = tile_modes(a.Ny, sizeof(Cplx<R>), sizeof(R));
   if (a.tile_modes > 0 && a.tile_modes < mb) mb = a.tile_modes;
   const size_t sm = (size_t)a.Ny * mb * (sizeof(Cplx<R>) + sizeof(R));
   const int nm = a.Mh;  // tiles start at m = 0
   const bool pdl = (a.pdl & 2) != 0;
-  if constexpr (sizeof(R) == 4) {
+  {
     if (a.tile_tma && a.mtma && mb == 8 && a.tile_threads <= 256 && !a.tile_cluster) {
       const size_t sm3 = modes_tma_pivot_offset(a.Ny) + (size_t)a.Ny * 32 + 128;
       return launch_ex(pdl, k_modes_tile_tma, dim3((nm + 7) / 8), dim3(kTileThreads), sm3, s, a, *a.mtma);
@@ -1478,13 +1527,11 @@ cudaError_t launch_modes(const PoissonArgs& a, cudaStream_t s) {
   }
 }
 
-template <class R>
 size_t row_smem(int Nx) {
   const int L = Nx / 2, T = (L >= 4) ? L / 4 : 1, rows = 256 / T;
-  return ((size_t)Nx + 2 * (size_t)rows * row_len_padded(L)) * sizeof(Cplx<R>);
+  return ((size_t)Nx + 2 * (size_t)rows * row_len_padded(L)) * sizeof(Cplx<float>);
 }
 
-template <class R>
 int row_blocks(int Nx, int Ny) {
   const int L = Nx / 2, T = (L >= 4) ? L / 4 : 1, rows = 256 / T;
   return (Ny + rows - 1) / rows;
@@ -1495,10 +1542,12 @@ cudaError_t poisson_t(const PoissonArgs& a, cudaStream_t s, cudaStream_t side, c
                       const cudaEvent_t* marks) {
   const bool warp_fft = (sizeof(R) == 4) && fftw_supported(a.Nx);
   cudaError_t e;
-  if (warp_fft) {
+  if constexpr (sizeof(R) == 8) {
+    e = launch_rfft64(a, s);
+  } else if (warp_fft) {
     e = launch_rfft_warp(a, s);
   } else {
-    k_rfft_rows<R><<<row_blocks<R>(a.Nx, a.Ny), 256, row_smem<R>(a.Nx), s>>>(a);
+    k_rfft_rows<<<row_blocks(a.Nx, a.Ny), 256, row_smem(a.Nx), s>>>(a);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) return e;
@@ -1506,37 +1555,48 @@ cudaError_t poisson_t(const PoissonArgs& a, cudaStream_t s, cudaStream_t side, c
   // solve, [2] after the inverse FFT (all on s); [3], [4] around the mean mode
   auto mark = [&](int k, cudaStream_t st) { return marks ? cudaEventRecord(marks[k], st) : cudaSuccess; };
   if ((e = mark(0, s)) != cudaSuccess) return e;
-  if (side) {
-    if ((e = cudaEventRecord(fork, s)) != cudaSuccess) return e;
-    if ((e = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess) return e;
+  if (sizeof(R) == 8 && a.y_solver != 1) {
+    if ((e = mark(3, s)) != cudaSuccess) return e;
+    if ((e = launch_modes64(a, s)) != cudaSuccess) return e;
+    if ((e = mark(4, s)) != cudaSuccess) return e;
+    side = nullptr;
+  } else {
+    if (side) {
+      if ((e = cudaEventRecord(fork, s)) != cudaSuccess) return e;
+      if ((e = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess) return e;
+    }
+    const cudaStream_t ms = side ? side : s;
+    if ((e = mark(3, ms)) != cudaSuccess) return e;
+    const size_t msm = 2 * (size_t)a.Ny * sizeof(typename MeanNum<R>::T);
+    if (a.Ny <= kMeanSmallRows)
+      k_mean_mode<R, kMeanThreadsSmall><<<1, kMeanThreadsSmall, msm, ms>>>(a);
+    else
+      k_mean_mode<R, kMeanThreads><<<1, kMeanThreads, msm, ms>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = mark(4, ms)) != cudaSuccess) return e;
+    if (side && (e = cudaEventRecord(join, side)) != cudaSuccess) return e;
+    e = (a.y_solver == 1) ? launch_modes_oddext(a, sizeof(R) == 8, s) : launch_modes(a, s);
+    if (e != cudaSuccess) return e;
   }
-  const cudaStream_t ms = side ? side : s;
-  if ((e = mark(3, ms)) != cudaSuccess) return e;
-  const size_t msm = 2 * (size_t)a.Ny * sizeof(typename MeanNum<R>::T);
-  if (a.Ny <= kMeanSmallRows)
-    k_mean_mode<R, kMeanThreadsSmall><<<1, kMeanThreadsSmall, msm, ms>>>(a);
-  else
-    k_mean_mode<R, kMeanThreads><<<1, kMeanThreads, msm, ms>>>(a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = mark(4, ms)) != cudaSuccess) return e;
-  if (side && (e = cudaEventRecord(join, side)) != cudaSuccess) return e;
-  e = (a.y_solver == 1) ? launch_modes_oddext(a, sizeof(R) == 8, s) : launch_modes<R>(a, s);
-  if (e != cudaSuccess) return e;
   if ((e = mark(1, s)) != cudaSuccess) return e;
-  if (warp_fft) {
+  if constexpr (sizeof(R) == 8) {
+    e = launch_irfft64(a, false, s);
+  } else if (warp_fft) {
     e = launch_irfft_warp(a, s);
   } else {
-    k_irfft_rows<R><<<row_blocks<R>(a.Nx, a.Ny), 256, row_smem<R>(a.Nx), s>>>(a);
+    k_irfft_rows<><<<row_blocks(a.Nx, a.Ny), 256, row_smem(a.Nx), s>>>(a);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) return e;
   if (a.ex) {
     // spectral E_x: the inverse row transform of -i k_m phi_m, formed as it
     // reads the solved spectrum
-    if (warp_fft) {
+    if constexpr (sizeof(R) == 8) {
+      e = launch_irfft64(a, true, s);
+    } else if (warp_fft) {
       e = launch_irfft_warp_dx(a, s);
     } else {
-      k_irfft_rows<R, true><<<row_blocks<R>(a.Nx, a.Ny), 256, row_smem<R>(a.Nx), s>>>(a);
+      k_irfft_rows<true><<<row_blocks(a.Nx, a.Ny), 256, row_smem(a.Nx), s>>>(a);
       e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;
@@ -1563,9 +1623,6 @@ template <class R>
 cudaError_t set_attrs_t() {
   cudaError_t e;
 
-  if ((e = allow_max_dynamic_smem(k_rfft_rows<R>)) != cudaSuccess) return e;
-  if ((e = allow_max_dynamic_smem(k_irfft_rows<R>)) != cudaSuccess) return e;
-  if ((e = allow_max_dynamic_smem(k_irfft_rows<R, true>)) != cudaSuccess) return e;
   if ((e = allow_max_dynamic_smem(k_mean_mode<R, kMeanThreads>)) != cudaSuccess) return e;
   if ((e = allow_max_dynamic_smem(k_mean_mode<R, kMeanThreadsSmall>)) != cudaSuccess) return e;
   if constexpr (sizeof(R) == 4) {
@@ -1578,10 +1635,17 @@ cudaError_t set_attrs_t() {
     if ((e = allow_max_dynamic_smem(k_modes_tile<R, 4, 1024>)) != cudaSuccess) return e;
     if ((e = allow_max_dynamic_smem(k_modes_tile<R, 2, 1024>)) != cudaSuccess) return e;
   }
-  if ((e = allow_max_dynamic_smem(k_modes_tile<R, 8>)) != cudaSuccess) return e;
-  if ((e = allow_max_dynamic_smem(k_modes_tile<R, 4>)) != cudaSuccess) return e;
-  if ((e = allow_max_dynamic_smem(k_modes_tile<R, 2>)) != cudaSuccess) return e;
-  return allow_max_dynamic_smem(k_modes_tile<R, 1>);
+  if constexpr (sizeof(R) == 8) {
+    if ((e = allow_max_dynamic_smem(k_modes64<8>)) != cudaSuccess) return e;
+    if ((e = allow_max_dynamic_smem(k_modes64<4>)) != cudaSuccess) return e;
+    if ((e = allow_max_dynamic_smem(k_modes64<2>)) != cudaSuccess) return e;
+    return allow_max_dynamic_smem(k_modes64<1>);
+  } else {
+    if ((e = allow_max_dynamic_smem(k_modes_tile<R, 8>)) != cudaSuccess) return e;
+    if ((e = allow_max_dynamic_smem(k_modes_tile<R, 4>)) != cudaSuccess) return e;
+    if ((e = allow_max_dynamic_smem(k_modes_tile<R, 2>)) != cudaSuccess) return e;
+    return allow_max_dynamic_smem(k_modes_tile<R, 1>);
+  }
 }
 
 template <class S, class R>
@@ -1620,9 +1684,8 @@ cudaError_t poisson_set_attributes() {
   return set_attrs_t<float>();
 }
 
-cudaError_t launch_rhoc(const void* g, long long plane, int storage, bool real_f64, int Nx, int Ny, int P,
-                        const float* rch, void* rhoc, cudaStream_t s) {
-  if (real_f64) return storage == 0 ? rhoc_t<double, double>(g, plane, Nx, Ny, P, rch, rhoc, s) : cudaErrorInvalidValue;
+cudaError_t launch_rhoc(const void* g, long long plane, int storage, int Nx, int Ny, int P, const float* rch,
+                        void* rhoc, cudaStream_t s) {
   switch (storage) {
     case 0: return rhoc_t<double, float>(g, plane, Nx, Ny, P, rch, rhoc, s);
     case 1: return rhoc_t<float, float>(g, plane, Nx, Ny, P, rch, rhoc, s);
