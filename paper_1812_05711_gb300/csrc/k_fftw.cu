@@ -9,81 +9,11 @@
 // W_L^(n1 k2), the warp transposes through shared memory (padded rows), and
 // lane k2 finishes with a 32-point FFT in registers.  No CTA-wide barrier.
 // The inverse uses IFFT(Z) = conj(FFT(conj(Z))) / L.
-#include <cmath>
-
-#include "ehd_dev.cuh"
+#include "fft_dev.cuh"
 
 namespace ehd {
 
 namespace {
-
-__constant__ float2 c_w32[32];  // exp(-2 pi i k / 32)
-__constant__ float2 c_w64[64];  // exp(-2 pi i k / 64)
-
-__host__ __device__ constexpr int bitrev(int i, int n) {
-  int r = 0;
-  for (int b = 1; b < n; b <<= 1) {
-    r = (r << 1) | (i & 1);
-    i >>= 1;
-  }
-  return r;
-}
-
-// in-register radix-2 FFT of length M <= 32 (forward, natural order in/out);
-// every index is a compile-time constant so the arrays stay in registers
-template <int M, int LEN>
-struct FftStage {
-  __device__ __forceinline__ static void run(float (&re)[M], float (&im)[M]) {
-#pragma unroll
-    for (int b = 0; b < M / LEN; ++b) {
-#pragma unroll
-      for (int k = 0; k < LEN / 2; ++k) {
-        const float2 w = c_w32[k * (32 / LEN)];
-        const int u = b * LEN + k, v = u + LEN / 2;
-        const float tr = re[v] * w.x - im[v] * w.y;
-        const float ti = re[v] * w.y + im[v] * w.x;
-        // the pair's sum and difference as packed two-float adds
-        const float2 a = make_float2(re[u], im[u]);
-        const float2 lo = __fadd2_rn(a, make_float2(-tr, -ti)), hi = __fadd2_rn(a, make_float2(tr, ti));
-        re[v] = lo.x;
-        im[v] = lo.y;
-        re[u] = hi.x;
-        im[u] = hi.y;
-      }
-    }
-    FftStage<M, LEN * 2>::run(re, im);
-  }
-};
-template <int M>
-struct FftStage<M, M * 2> {
-  __device__ __forceinline__ static void run(float (&)[M], float (&)[M]) {}
-};
-
-template <int M>
-__device__ __forceinline__ void fft_reg(float (&re)[M], float (&im)[M]) {
-#pragma unroll
-  for (int i = 0; i < M; ++i) {
-    const int j = bitrev(i, M);
-    if (j > i) {
-      const float tr = re[i], ti = im[i];
-      re[i] = re[j];
-      im[i] = im[j];
-      re[j] = tr;
-      im[j] = ti;
-    }
-  }
-  FftStage<M, 2>::run(re, im);
-}
-
-__device__ __forceinline__ float2 cm(float2 a, float2 b) {
-  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-
-__device__ __forceinline__ void two_sum_f(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
-}
 
 // Four-step forward FFT of rows of L = 32 E complex values, R <= 32 / E rows
 // per warp (R = 32 / E: every lane works in both stages).  First stage, per row r:
@@ -93,20 +23,6 @@ __device__ __forceinline__ void two_sum_f(float a, float b, float& s, float& e) 
 // and finishes with a 32-point FFT, holding X_r[k2 + E k1] in (ore[k1],
 // oim[k1]).  Per row the arithmetic is that of the one-row-per-warp form.
 // tw: exp(-2 pi i q / N) for q < N (global).
-
-// the first stage's twiddles of lane n1: powers of W_N^(2 n1), resynchronised
-// from the table every 4 steps
-template <int E>
-__device__ __forceinline__ void four_step_twiddles(const float2* __restrict__ tw, int lane, float2 (&w)[E]) {
-  constexpr int N = 64 * E;
-  const float2 base = tw[(2 * lane) & (N - 1)];
-  float2 c = make_float2(1.0f, 0.0f);
-#pragma unroll
-  for (int k2 = 0; k2 < E; ++k2) {
-    if (k2 > 0) c = ((k2 & 3) == 0) ? tw[(2 * lane * k2) & (N - 1)] : cm(c, base);
-    w[k2] = c;
-  }
-}
 
 template <int E>
 __device__ __forceinline__ void four_step_first(float (&re)[E], float (&im)[E], const float2 (&w)[E], float2* sm,
@@ -582,27 +498,124 @@ __global__ void __launch_bounds__(kCtaT, 12) k_irfft_cta(PoissonArgs a) {
       dphi2[k1 + 16 * (4 * q + i) + 256 * d] = make_float2(zr[4 * d + i] * inL, -zi[4 * d + i] * inL);
 }
 
+// The same transforms of one row with all lanes at work (LaneFft): the single
+// run's rows of up to 512 reals, bound by the length of one warp's instruction
+// chain.  The same bits as rfft_warp_rows / irfft_warp_rows.
+template <int E>
+__device__ __forceinline__ void rfft_lane_row(const PoissonArgs& a, int y, const LaneFft<E>& fft,
+                                              const float2 (&wk)[E], float2* sm) {
+  const int lane = threadIdx.x & 31;
+  constexpr int L = 32 * E, N = 2 * L;
+  const float nieps = -(float)a.inv_eps;
+  const float2* rc2 = reinterpret_cast<const float2*>(static_cast<const float*>(a.rhoc) + (long long)y * a.P);
+  const float *rdn, *rup;
+  rhoc_partials<float>(a, y, rdn, rup);
+  float2 v[E];
+#pragma unroll
+  for (int n2 = 0; n2 < E; ++n2) {
+    v[n2] = rc2[lane + 32 * n2];
+    if (rdn) {
+      const float2 d = reinterpret_cast<const float2*>(rdn)[lane + 32 * n2];
+      v[n2].x += d.x;
+      v[n2].y += d.y;
+    }
+    if (rup) {
+      const float2 u = reinterpret_cast<const float2*>(rup)[lane + 32 * n2];
+      v[n2].x += u.x;
+      v[n2].y += u.y;
+    }
+  }
+  const float c0 = __shfl_sync(0xffffffffu, v[0].x, 0);  // the row constant (see rfft_warp_rows)
+  float re[E], im[E];
+#pragma unroll
+  for (int n2 = 0; n2 < E; ++n2) {
+    re[n2] = (v[n2].x - c0) * nieps;
+    im[n2] = (v[n2].y - c0) * nieps;
+  }
+  fft.run(re, im, lane);
+  if (lane == 0)
+    static_cast<float2*>(a.spec0)[y] = mean_coefficient(make_float2(re[0], im[0]), c0, nieps, (float)N);
+  lane_fft_store<E>(re, im, sm, lane);
+  float2* spec = static_cast<float2*>(a.spec) + (long long)y * a.Mp;
+#pragma unroll
+  for (int j = 0; j < E; ++j) {
+    const int k = lane + 32 * j;
+    spec[k] = (k == 0) ? make_float2(0.0f, 0.0f) : untangle<E>(sm, k, wk[j]);
+  }
+  if (lane == 0) spec[L] = make_float2(re[0] - im[0], 0.0f);  // Nyquist: Re Z0 - Im Z0
+}
+
+template <int E, bool DX>
+__device__ __forceinline__ void irfft_lane_row(const PoissonArgs& a, int y, const LaneFft<E>& fft,
+                                               const float2 (&wk)[E], float2* sm) {
+  const int lane = threadIdx.x & 31;
+  constexpr int L = 32 * E;
+  const float2* spec = static_cast<const float2*>(a.spec) + (long long)y * a.Mp;
+  float re[E], im[E];
+#pragma unroll
+  for (int n2 = 0; n2 < E; ++n2) {
+    const int k = lane + 32 * n2;
+    const float2 sk = (k == 0) ? make_float2(0.0f, 0.0f) : spec_in<DX>(spec, k, L);
+    const float2 z = entangle(sk, spec_in<DX>(spec, L - k, L), wk[n2]);
+    re[n2] = z.x;
+    im[n2] = z.y;
+  }
+  fft.run(re, im, lane);
+  lane_fft_store<E>(re, im, sm, lane);
+  float2* out = reinterpret_cast<float2*>(static_cast<float*>(DX ? a.ex : a.dphi) + (long long)y * a.P);
+  const float inL = 1.0f / (float)L;
+#pragma unroll
+  for (int j = 0; j < E; ++j) {
+    const float2 v = sm[lpad(lane + 32 * j)];
+    out[lane + 32 * j] = make_float2(v.x * inL, -v.y * inL);
+  }
+}
+
 // one warp per row: a single run's transforms are bound by latency, and
 // more warps in flight beat fuller ones (128 x 104: 16.1 against 28.7 us
 // per step with 32/E rows per warp)
 template <int E>
 __global__ void __launch_bounds__(128) k_rfft_warp(PoissonArgs a) {
-  __shared__ float2 smem[4][E * 33];
-  grid_dep_wait();
-  grid_dep_launch();
+  __shared__ float2 smem[4][E * 34];
   const int warp = threadIdx.x >> 5;
   const int y = blockIdx.x * 4 + warp;
-  if (y < a.Ny) rfft_warp_rows<E, 1>(a, y, smem[warp]);
+  if constexpr (E <= 8) {
+    // constant tables before the wait for the step kernel
+    LaneFft<E> fft;
+    float2 wk[E];
+    fft.init(static_cast<const float2*>(a.tw), threadIdx.x & 31);
+    untangle_factors<E>(static_cast<const float2*>(a.tw), threadIdx.x & 31, wk);
+    grid_dep_wait();
+    grid_dep_launch();
+    if (y < a.Ny) rfft_lane_row<E>(a, y, fft, wk, smem[warp]);
+  } else {
+    grid_dep_wait();
+    grid_dep_launch();
+    if (y < a.Ny) rfft_warp_rows<E, 1>(a, y, smem[warp]);
+  }
 }
 
 template <int E, bool DX = false>
 __global__ void __launch_bounds__(128) k_irfft_warp(PoissonArgs a) {
-  __shared__ float2 smem[4][E * 33];
-  grid_dep_wait();
-  grid_dep_launch();
+  __shared__ float2 smem[4][E * 34];
   const int warp = threadIdx.x >> 5;
   const int y = blockIdx.x * 4 + warp;
-  if (y < a.Ny) irfft_warp_rows<E, 1, DX>(a, y, smem[warp]);
+  if constexpr (E <= 8) {
+    const float2* __restrict__ tw = static_cast<const float2*>(a.tw);
+    LaneFft<E> fft;
+    float2 wk[E];
+    fft.init(tw, threadIdx.x & 31);
+    // W_N^k for k = lane + 32 n2
+#pragma unroll
+    for (int n2 = 0; n2 < E; ++n2) wk[n2] = cmf1(tw[threadIdx.x & 31], tw[32 * n2]);
+    grid_dep_wait();
+    grid_dep_launch();
+    if (y < a.Ny) irfft_lane_row<E, DX>(a, y, fft, wk, smem[warp]);
+  } else {
+    grid_dep_wait();
+    grid_dep_launch();
+    if (y < a.Ny) irfft_warp_rows<E, 1, DX>(a, y, smem[warp]);
+  }
 }
 
 // Batch: warps of a fixed grid take row items (run, y0: the run's rows y0 ..
@@ -690,15 +703,7 @@ cudaError_t launch_batch_irfft(const BatchTables& t, int step, int grid, cudaStr
   return e;
 }
 
-cudaError_t fftw_set_tables() {
-  float2 w32[32], w64[64];
-  const double pi = 3.141592653589793238462643383279502884;
-  for (int k = 0; k < 32; ++k) w32[k] = make_float2((float)std::cos(2 * pi * k / 32), (float)-std::sin(2 * pi * k / 32));
-  for (int k = 0; k < 64; ++k) w64[k] = make_float2((float)std::cos(2 * pi * k / 64), (float)-std::sin(2 * pi * k / 64));
-  cudaError_t e = cudaMemcpyToSymbol(c_w32, w32, sizeof w32);
-  if (e != cudaSuccess) return e;
-  return cudaMemcpyToSymbol(c_w64, w64, sizeof w64);
-}
+cudaError_t fftw_set_tables() { return fft_set_tables(); }
 
 bool fftw_supported(int Nx) { return Nx >= 64 && Nx <= 2048; }
 
