@@ -111,9 +111,9 @@ cudaError_t tma_encode_2d(CUtensorMap* m, const void* base, unsigned long long i
                           unsigned long long row_bytes, unsigned box_inner, unsigned box_outer);
 cudaError_t modes_tma_encode(ModesTma* t, const void* spec, const void* rfac, int Ny, int Mp);
 
-// Constants of the FP64 collision (collide_f64), formed on the host: an FP64
-// instruction takes its constant operand from the kernel parameters, and no
-// thread spends FP64 issue slots on forming one.
+// Constants of the FP64 collision (collide_f64).  The one-node-per-thread step
+// takes them from the host: an FP64 instruction reads its constant operand from
+// the kernel parameters, and no thread spends FP64 issue slots on forming one.
 struct CollideF64 {
   double hp, hm;        // (1 - omega+) / 2, (1 - omega-) / 2
   double rw;            // W1 omega+
@@ -122,7 +122,7 @@ struct CollideF64 {
   double ghp, ghm;      // (1 - omega_g+) / 2, (1 - omega_g-) / 2
   double grw, gg, gjm;  // W1 omega_g+, 4.5 W1 omega_g+, 3 W1 omega_g-
 };
-inline CollideF64 collide_f64_constants(double wp, double wm, double gwp, double gwm) {
+__host__ __device__ inline CollideF64 collide_f64_constants(double wp, double wm, double gwp, double gwm) {
   CollideF64 k;
   k.hp = 0.5 * (1.0 - wp);
   k.hm = 0.5 * (1.0 - wm);
@@ -168,7 +168,6 @@ struct StepArgs {
   int cols_per_lane;         // 1: 32-column strips (30 owned); 2: 64-column strips (60 owned)
   int pdl;                   // launch with programmatic dependent launch (see launch_ex)
   const float* base_tab;     // perturbation form: the march table of time t ([Ny][4]); nullptr otherwise
-  CollideF64 k64;            // constants of the FP64 collision
 };
 
 // -------------------------------------------------- FP64 TRT collision ---
@@ -494,6 +493,11 @@ int oddext_factors(int n, int* fac, int cap);
 size_t oddext_smem_bytes(int NE, bool real_f64);
 cudaError_t launch_modes_oddext(const PoissonArgs& a, bool real_f64, cudaStream_t s);
 cudaError_t oddext_set_attributes();
+// Many steps of a small FP32 run in one launch with its state on chip
+// (k_resident.cu): whether the size fits a cluster of this GPU (also sets the
+// kernel's attributes), and `steps` steps from a.fin / a.gin back into them.
+bool resident_supported(int Nx, int Ny, int storage);
+cudaError_t launch_resident(const StepArgs& a, const PoissonArgs& pa, int storage, int steps, cudaStream_t s);
 // rho_c = sum_i g_i (+ the row shift) into the charge plane (FP32 compute).
 cudaError_t launch_rhoc(const void* g, long long plane, int storage, int Nx, int Ny, int P,
                         const float* rch, void* rhoc, cudaStream_t s);

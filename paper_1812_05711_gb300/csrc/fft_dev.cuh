@@ -12,7 +12,30 @@ namespace ehd {
 
 static __constant__ float2 c_w32[32];  // exp(-2 pi i k / 32)
 static __constant__ float2 c_w64[64];  // exp(-2 pi i k / 64)
-static __device__ float2 g_w64[64];    // the same, for lane-dependent indices
+// the second one rounded to FP32, in global memory for lane-dependent indices
+static __device__ float2 g_w64[64] = {
+    {1.0f, -0.0f}, {0.99518472f, -0.0980171412f}, {0.980785251f, -0.195090324f},
+    {0.956940353f, -0.290284663f}, {0.923879504f, -0.382683426f}, {0.881921291f, -0.471396744f},
+    {0.831469595f, -0.555570245f}, {0.773010433f, -0.634393275f}, {0.707106769f, -0.707106769f},
+    {0.634393275f, -0.773010433f}, {0.555570245f, -0.831469595f}, {0.471396744f, -0.881921291f},
+    {0.382683426f, -0.923879504f}, {0.290284663f, -0.956940353f}, {0.195090324f, -0.980785251f},
+    {0.0980171412f, -0.99518472f}, {6.12323426e-17f, -1.0f}, {-0.0980171412f, -0.99518472f},
+    {-0.195090324f, -0.980785251f}, {-0.290284663f, -0.956940353f}, {-0.382683426f, -0.923879504f},
+    {-0.471396744f, -0.881921291f}, {-0.555570245f, -0.831469595f}, {-0.634393275f, -0.773010433f},
+    {-0.707106769f, -0.707106769f}, {-0.773010433f, -0.634393275f}, {-0.831469595f, -0.555570245f},
+    {-0.881921291f, -0.471396744f}, {-0.923879504f, -0.382683426f}, {-0.956940353f, -0.290284663f},
+    {-0.980785251f, -0.195090324f}, {-0.99518472f, -0.0980171412f}, {-1.0f, -1.22464685e-16f},
+    {-0.99518472f, 0.0980171412f}, {-0.980785251f, 0.195090324f}, {-0.956940353f, 0.290284663f},
+    {-0.923879504f, 0.382683426f}, {-0.881921291f, 0.471396744f}, {-0.831469595f, 0.555570245f},
+    {-0.773010433f, 0.634393275f}, {-0.707106769f, 0.707106769f}, {-0.634393275f, 0.773010433f},
+    {-0.555570245f, 0.831469595f}, {-0.471396744f, 0.881921291f}, {-0.382683426f, 0.923879504f},
+    {-0.290284663f, 0.956940353f}, {-0.195090324f, 0.980785251f}, {-0.0980171412f, 0.99518472f},
+    {-1.83697015e-16f, 1.0f}, {0.0980171412f, 0.99518472f}, {0.195090324f, 0.980785251f},
+    {0.290284663f, 0.956940353f}, {0.382683426f, 0.923879504f}, {0.471396744f, 0.881921291f},
+    {0.555570245f, 0.831469595f}, {0.634393275f, 0.773010433f}, {0.707106769f, 0.707106769f},
+    {0.773010433f, 0.634393275f}, {0.831469595f, 0.555570245f}, {0.881921291f, 0.471396744f},
+    {0.923879504f, 0.382683426f}, {0.956940353f, 0.290284663f}, {0.980785251f, 0.195090324f},
+    {0.99518472f, 0.0980171412f}};
 
 __host__ __device__ constexpr int bitrev(int i, int n) {
   int r = 0;
@@ -224,8 +247,7 @@ static cudaError_t fft_set_tables() {
   for (int k = 0; k < 64; ++k) w64[k] = make_float2((float)std::cos(2 * pi * k / 64), (float)-std::sin(2 * pi * k / 64));
   cudaError_t e = cudaMemcpyToSymbol(c_w32, w32, sizeof w32);
   if (e != cudaSuccess) return e;
-  if ((e = cudaMemcpyToSymbol(c_w64, w64, sizeof w64)) != cudaSuccess) return e;
-  return cudaMemcpyToSymbol(g_w64, w64, sizeof w64);
+  return cudaMemcpyToSymbol(c_w64, w64, sizeof w64);
 }
 
 }  // namespace ehd

@@ -26,54 +26,11 @@
 // halo row below and above the slab collided but not stored.
 #include <type_traits>
 
-#include "ehd_dev.cuh"
+#include "march_dev.cuh"
 
 namespace ehd {
 
 namespace {
-
-template <class R>
-__device__ __forceinline__ void trt_f2(R& fi, R& fo, R w, R drho, R rho, R cu, R usq15, R cF, R uF3, R wp, R wm, R cp,
-                                       R cm) {
-  const R ep = w * (drho + rho * (R(4.5) * cu * cu - usq15));
-  const R em = w * rho * R(3) * cu;
-  const R Fp = w * (R(9) * cu * cF - uF3);
-  const R Fm = w * R(3) * cF;
-  const R sp = R(0.5) * (fi + fo), sm = R(0.5) * (fi - fo);
-  const R A = cp * Fp - wp * (sp - ep);
-  const R B = cm * Fm - wm * (sm - em);
-  fi = fi + A + B;
-  fo = fo + A - B;
-}
-
-// trt_f2 for a pair that crosses rows (fi moves up, fo down) in storage
-// shifted by a density ramp r(y) = r(0) + dr y: with dq = -dr / omega- the
-// antisymmetric part hands fi its storage offset change -w dr and fo +w dr,
-// at no extra instruction (dq is added inside the product w (3 rho cu + dq)).
-template <class R>
-__device__ __forceinline__ void trt_f2y(R& fi, R& fo, R w, R drho, R rho, R cu, R usq15, R cF, R uF3, R wp, R wm,
-                                        R cp, R cm, R dq) {
-  const R ep = w * (drho + rho * (R(4.5) * cu * cu - usq15));
-  const R em = w * (rho * R(3) * cu + dq);
-  const R Fp = w * (R(9) * cu * cF - uF3);
-  const R Fm = w * R(3) * cF;
-  const R sp = R(0.5) * (fi + fo), sm = R(0.5) * (fi - fo);
-  const R A = cp * Fp - wp * (sp - ep);
-  const R B = cm * Fm - wm * (sm - em);
-  fi = fi + A + B;
-  fo = fo + A - B;
-}
-
-template <class R>
-__device__ __forceinline__ void trt_g2(R& gi, R& go, R w, R drc, R rc, R cv, R vsq15, R wp, R wm) {
-  const R ep = w * (drc + rc * (R(4.5) * cv * cv - vsq15));
-  const R em = w * rc * R(3) * cv;
-  const R sp = R(0.5) * (gi + go), sm = R(0.5) * (gi - go);
-  const R A = -wp * (sp - ep);
-  const R B = -wm * (sm - em);
-  gi = gi + A + B;
-  go = go + A - B;
-}
 
 // cp.async of one element (4 or 8 bytes) global -> shared, per thread
 template <int BYTES>
@@ -465,41 +422,6 @@ struct March2Stages {
   static constexpr size_t kBytesPerWarp = (size_t)NSTAGE * kSlots * 32 * kSlotBytes;
 };
 
-template <class S, class R>
-__device__ __forceinline__ void collide_node(R (&f)[9], R (&g)[9], R Ex, R Ey, R sy, R sf, R dq, R mub, R wp, R wm,
-                                             R cp, R cm, R gwp, R gwm, const CollideF64& k64, bool& bad) {
-  if constexpr (sizeof(R) == 8) {  // unshifted: sy, sf and dq are zero
-    collide_f64(f, g, Ex, Ey, mub, k64, bad);
-    return;
-  }
-  const R W0 = (R)kW0, W1 = (R)kW1, W2 = (R)kW2;
-  const R drho = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
-  const R rho = sf + drho;
-  const R jx = (f[1] - f[3]) + (f[5] - f[7]) + (f[8] - f[6]);
-  const R jy = (f[2] - f[4]) + (f[5] - f[7]) + (f[6] - f[8]);
-  const R drc = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
-  const R rc = sy + drc;
-  bad = !isfinite(drho) || !isfinite(drc);
-  const R Fx = rc * Ex, Fy = rc * Ey;
-  const R irho = R(1) / rho;
-  const R ux = (jx + R(0.5) * Fx) * irho;
-  const R uy = (jy + R(0.5) * Fy) * irho;
-  const R vx = ux + mub * Ex, vy = uy + mub * Ey;
-  const R usq15 = R(1.5) * (ux * ux + uy * uy);
-  const R uF3 = R(3) * (ux * Fx + uy * Fy);
-  f[0] = f[0] - wp * (f[0] - W0 * (drho - rho * usq15)) - cp * W0 * uF3;
-  trt_f2<R>(f[1], f[3], W1, drho, rho, ux, usq15, Fx, uF3, wp, wm, cp, cm);
-  trt_f2y<R>(f[2], f[4], W1, drho, rho, uy, usq15, Fy, uF3, wp, wm, cp, cm, dq);
-  trt_f2y<R>(f[5], f[7], W2, drho, rho, ux + uy, usq15, Fx + Fy, uF3, wp, wm, cp, cm, dq);
-  trt_f2y<R>(f[6], f[8], W2, drho, rho, uy - ux, usq15, Fy - Fx, uF3, wp, wm, cp, cm, dq);
-  const R vsq15 = R(1.5) * (vx * vx + vy * vy);
-  g[0] = g[0] - gwp * (g[0] - W0 * (drc - rc * vsq15));
-  trt_g2<R>(g[1], g[3], W1, drc, rc, vx, vsq15, gwp, gwm);
-  trt_g2<R>(g[2], g[4], W1, drc, rc, vy, vsq15, gwp, gwm);
-  trt_g2<R>(g[5], g[7], W2, drc, rc, vx + vy, vsq15, gwp, gwm);
-  trt_g2<R>(g[6], g[8], W2, drc, rc, vy - vx, vsq15, gwp, gwm);
-}
-
 // Perturbation form (FP32 compute): the fluid part as collide_node, with the
 // full field E = E_B + E' in the force; the charge populations g are the
 // departures d = g - B_g(y) from the x-uniform base state, and their TRT
@@ -727,8 +649,8 @@ __device__ __forceinline__ void march2_body(const StepArgs& a, int strip, int sl
       collide_node_pert<R>(f0, g0, Ex0, EB + Ey0, Ey0, sy, uBy, vby, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, b0);
       collide_node_pert<R>(f1, g1, Ex1, EB + Ey1, Ey1, sy, uBy, vby, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, b1);
     } else {
-      collide_node<S, R>(f0, g0, Ex0, Ey0, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, a.k64, b0);
-      collide_node<S, R>(f1, g1, Ex1, Ey1, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, a.k64, b1);
+      collide_node<S, R>(f0, g0, Ex0, Ey0, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, b0);
+      collide_node<S, R>(f1, g1, Ex1, Ey1, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, b1);
     }
     if (owned && (b0 || b1)) bad = true;
     // pulled values at (xc, xc + 1): x-shift by c_x
@@ -1277,8 +1199,8 @@ __device__ __forceinline__ void march_tma_body(const StepArgs& a, const MarchTma
       g1[i] = G[i][1];
     }
     bool b0, b1;
-    collide_node<float, R>(f0, g0, Ex0, Ey0, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, a.k64, b0);
-    collide_node<float, R>(f1, g1, Ex1, Ey1, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, a.k64, b1);
+    collide_node<float, R>(f0, g0, Ex0, Ey0, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, b0);
+    collide_node<float, R>(f1, g1, Ex1, Ey1, sy, sf, fdq, mub, wp, wm, cp, cm, gwp, gwm, b1);
     if (owned && (b0 || b1)) bad = true;
     const R P1f0 = from_left(f1[1]), P5f0 = from_left(f1[5]), P8f0 = from_left(f1[8]);
     const R P3f1 = from_right(f0[3]), P6f1 = from_right(f0[6]), P7f1 = from_right(f0[7]);

@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(kStepThreads) k_step(StepArgs a, int rows) {
 // CTAs and eight with four; the loads of up to 16 resident warps overlap the
 // arithmetic).  FP64 storage is unshifted (rch == nullptr, fb = fd = 0).
 constexpr int kStep64Threads = 32;
-__global__ void __launch_bounds__(kStep64Threads, 16) k_step64(StepArgs a) {
+__global__ void __launch_bounds__(kStep64Threads, 16) k_step64(StepArgs a, CollideF64 k64) {
   const int x = blockIdx.x * kStep64Threads + threadIdx.x, y = blockIdx.y;
   const int Nx = a.Nx, Ny = a.Ny, P = a.P;
   const long long pl = a.plane;
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kStep64Threads, 16) k_step64(StepArgs a) {
     const double Ex = -0.5 * (pE - pW);
     const double Ey = fma(-0.5, pN - pS, __ldg(static_cast<const double*>(a.Ebar) + y));
     bool bad;
-    collide_f64(f, g, Ex, Ey, a.mub, a.k64, bad);
+    collide_f64(f, g, Ex, Ey, a.mub, k64, bad);
     if (bad) atomicOr(a.err, 1);
     // streaming: f_i(x + c_i, t + 1) = f_i*(x, t)
     const long long yo = (long long)y * P;
@@ -339,7 +339,7 @@ cudaError_t launch_step(const StepArgs& a, int storage, bool real_f64, int rows,
   if (real_f64) {
     if (storage != 0) return cudaErrorInvalidValue;
     return launch_ex((a.pdl & 8) != 0, k_step64, dim3((a.Nx + kStep64Threads - 1) / kStep64Threads, a.Ny),
-                     dim3(kStep64Threads), 0, s, a);
+                     dim3(kStep64Threads), 0, s, a, collide_f64_constants(a.wp, a.wm, a.gwp, a.gwm));
   }
   switch (storage) {
     case 0: return step_t<double, float>(a, rows, s);
