@@ -397,8 +397,8 @@ void* ehd_batch_stream(ehd_batch* batch);
  * items fill about one wave), EHD_BATCH_MARCH_CTAS / EHD_BATCH_ROW_CTAS /
  * EHD_BATCH_TILE_CTAS (fixed grid of the persistent march, row-FFT and
  * wavenumber kernels), EHD_BATCH_PDL (a mask of the phase kernels launched
- * with programmatic dependent launch: 1 the forward transforms, the default,
- * 2 the wavenumber tiles, 4 the inverse transforms).  Drops the captured
+ * with programmatic dependent launch: 1 the forward transforms, 2 the
+ * wavenumber solves, 4 the inverse transforms; 5 by default).  Drops the captured
  * graphs.  EHD_EINVAL otherwise. */
 #define EHD_BATCH_SLAB_ROWS 1
 #define EHD_BATCH_MARCH_CTAS 2

@@ -163,7 +163,7 @@ struct ehd_batch {
   int2* d_rows = nullptr;
   int2* d_tiles = nullptr;
   int* d_counts = nullptr;
-  int* d_work = nullptr;  // [4] dynamic item counters of the step's phases
+  int* d_work = nullptr;  // [2] dynamic item counters of the step's march and y solves
   BatchRunDesc* h_runs = nullptr;
   int4* h_march = nullptr;
   int2* h_rows = nullptr;
@@ -174,10 +174,10 @@ struct ehd_batch {
   int grid_march = 0, grid_rows = 0, grid_tiles = 0, grid_mean = 0, modes_smem = 0;
   int slab_rows_fixed = 0;  // 0: choose from the membership
   // programmatic dependent launch of the phase kernels (mask: 1 forward
-  // transforms, 2 wavenumber tiles, 4 inverse transforms): the forward
-  // transforms only (64 uneven runs: 213.0 us per step against 214.3
-  // without, 213.5 with all three)
-  int pdl = 1;
+  // transforms, 2 wavenumber solves, 4 inverse transforms): both transforms
+  // (64 uneven runs: 200.8 us per step against 200.9 with the forward ones
+  // only and 202.6 with the solves too; 8 runs: 39.2, 39.9, 43.8)
+  int pdl = 5;
   std::map<int, cudaGraphExec_t> graphs;  // by 2 x tick length + (any member in the perturbation form)
 };
 
@@ -1419,6 +1419,7 @@ BatchTables batch_tables(const ehd_batch* b) {
   t.tile_items = b->d_tiles;
   t.counts = b->d_counts;
   t.work = b->d_work;
+  t.mean_in_modes = b->max_ny <= 1024;
   t.modes_smem = b->modes_smem;
   t.emax = std::max(1, b->max_nx / 64);
   t.pdl = b->pdl;
@@ -1457,14 +1458,19 @@ void batch_build_items(ehd_batch* b, int resident_warps) {
   std::vector<size_t> by_nx(nmem), by_ny(nmem);
   for (size_t i = 0; i < nmem; ++i) by_nx[i] = by_ny[i] = i;
   std::stable_sort(by_nx.begin(), by_nx.end(),
-                   [&](size_t p, size_t q) { return b->members[p]->Nx < b->members[q]->Nx; });
+                   [&](size_t p, size_t q) { return b->members[p]->Nx > b->members[q]->Nx; });
   std::stable_sort(by_ny.begin(), by_ny.end(),
                    [&](size_t p, size_t q) { return b->members[p]->Ny > b->members[q]->Ny; });
-  // row items: 2048 / Nx rows of one run each (one warp's four-step
-  // transform), the narrowest runs first: their items walk the most rows one
-  // after another, so they are the longest
-  for (size_t i : by_nx)
-    for (int y = 0; y < b->members[i]->Ny; y += 2048 / b->members[i]->Nx) b->h_rows[nr++] = make_int2((int)i, y);
+  // row items, the widest rows first (the longest): rows of up to 512 a few
+  // at a time, wider ones 2048 / Nx
+  long long rows_all = 0;
+  for (ehd_run* r : b->members) rows_all += r->Ny;
+  const long long row_warps = 4LL * b->grid_rows;
+  const int few = (int)std::max(1LL, std::min(4LL, rows_all / row_warps));
+  for (size_t i : by_nx) {
+    const int step = b->members[i]->Nx <= 512 ? few : 2048 / b->members[i]->Nx;
+    for (int y = 0; y < b->members[i]->Ny; y += step) b->h_rows[nr++] = make_int2((int)i, row_item(y, step));
+  }
   for (size_t i : by_ny)
     for (int m0 = 0; m0 < b->members[i]->Mh; m0 += kBatchTileModes) b->h_tiles[nt++] = make_int2((int)i, m0);
   b->h_counts[0] = (int)b->members.size();
@@ -1483,21 +1489,21 @@ ehd_status batch_capture(ehd_batch* b, int K, bool pert, cudaGraphExec_t* out) {
   EHD_CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
   for (int s = 0; s < K && e == cudaSuccess; ++s) {
-    e = cudaMemsetAsync(b->d_work, 0, 4 * sizeof(int), b->stream);
-    if (e == cudaSuccess) e = launch_batch_march(t, s, b->grid_march, pert, b->stream);
+    e = launch_batch_march(t, s, b->grid_march, pert, b->stream);
     if (e == cudaSuccess) e = launch_batch_rfft(t, s, b->grid_rows, b->stream);
-    if (e == cudaSuccess) e = cudaEventRecord(b->ev_fork, b->stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->ev_fork, 0);
+    const bool side = !t.mean_in_modes;
+    if (e == cudaSuccess && (side || pert)) e = cudaEventRecord(b->ev_fork, b->stream);
+    if (e == cudaSuccess && side) e = cudaStreamWaitEvent(b->side, b->ev_fork, 0);
     if (pert) {
       if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side2, b->ev_fork, 0);
       if (e == cudaSuccess) e = launch_batch_base(t, s, b->max_runs, b->max_ny, b->side2);
       if (e == cudaSuccess) e = cudaEventRecord(b->ev_base, b->side2);
     }
-    if (e == cudaSuccess) e = launch_batch_mean(t, s, b->grid_mean, b->side);
-    if (e == cudaSuccess) e = cudaEventRecord(b->ev_join, b->side);
+    if (e == cudaSuccess && side) e = launch_batch_mean(t, s, b->grid_mean, b->side);
+    if (e == cudaSuccess && side) e = cudaEventRecord(b->ev_join, b->side);
     if (e == cudaSuccess) e = launch_batch_modes(t, s, b->grid_tiles, b->stream);
     if (e == cudaSuccess) e = launch_batch_irfft(t, s, b->grid_rows, b->stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->ev_join, 0);
+    if (e == cudaSuccess && side) e = cudaStreamWaitEvent(b->stream, b->ev_join, 0);
     if (pert && e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->ev_base, 0);
   }
   cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
@@ -1575,7 +1581,7 @@ ehd_status ehd_batch_create(int max_runs, size_t hbm_budget, int max_nx, int max
   b->d_rows = devmem<int2>(b->cap_rows);
   b->d_tiles = devmem<int2>(b->cap_tiles);
   b->d_counts = devmem<int>(4);
-  b->d_work = devmem<int>(4);
+  b->d_work = devmem<int>(2);
   b->h_runs = pinned<BatchRunDesc>(max_runs);
   b->h_march = pinned<int4>(b->cap_march);
   b->h_rows = pinned<int2>(b->cap_rows);
@@ -1585,6 +1591,11 @@ ehd_status ehd_batch_create(int max_runs, size_t hbm_budget, int max_nx, int max
       !b->h_rows || !b->h_tiles || !b->h_counts) {
     batch_free(b);
     return fail(EHD_ENOMEM, "batch table allocation failed");
+  }
+  if (cudaMemsetAsync(b->d_work, 0, 2 * sizeof(int), b->stream) != cudaSuccess ||
+      cudaStreamSynchronize(b->stream) != cudaSuccess) {
+    batch_free(b);
+    return fail(EHD_ECUDA, "clearing the batch's counters failed");
   }
   const int wps = march_warps_per_sm(1, false, 2, 2);
   b->grid_march = b->sms * std::max(1, wps / 4);

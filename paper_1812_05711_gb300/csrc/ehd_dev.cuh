@@ -421,15 +421,21 @@ struct BatchRunDesc {
 struct BatchTables {
   const BatchRunDesc* runs;
   const int4* march_items;  // (run, strip, slab, 0)
-  const int2* row_items;    // (run, row)
+  const int2* row_items;    // (run, rows: row_item)
   const int2* tile_items;   // (run, first wavenumber)
   const int* counts;        // device: [0] runs, [1] march items, [2] rows, [3] tiles
-  int* work;                // device: items taken so far in this step's march, forward FFT,
-                            // wavenumber and inverse FFT phases (zeroed before each step)
+  int* work;                // device: [0] march items and [1] y solves taken from the step's counters (each
+                            // zeroed, for the next step, by the transform that follows its phase)
+  int mean_in_modes;        // the mean modes are items of the wavenumber kernel (all runs of at most 1024 rows)
   int modes_smem;           // tile bytes for the largest admissible Ny (fixed per batch)
   int pdl;                  // programmatic dependent launch: 1 forward transforms, 2 tiles, 4 inverse
   int emax;                 // largest admissible Nx / 64: the widest warp-FFT shape compiled in
 };
+
+// Rows of a row-transform item: first row and how many (Ny <= 4096).
+__host__ __device__ __forceinline__ int row_item(int y, int count) { return y | (count << 16); }
+__device__ __forceinline__ int row_item_row(int v) { return v & 0xffff; }
+__device__ __forceinline__ int row_item_count(int v) { return v >> 16; }
 
 // Dynamic scheduling of a batch phase's items (largest first in the lists):
 // one lane or thread takes the next index from the phase's counter.

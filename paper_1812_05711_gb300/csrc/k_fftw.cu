@@ -618,48 +618,75 @@ __global__ void __launch_bounds__(128) k_irfft_warp(PoissonArgs a) {
   }
 }
 
-// Batch: warps of a fixed grid take row items (run, y0: the run's rows y0 ..
-// y0 + 2048/Nx - 1); the row length picks the transform shape.
-// EMAX: the widest row shape of the batch (Nx / 64); narrower batches get an
-// instance with fewer registers (the inverse up to EMAX = 8 at most 102:
-// five CTAs per SM), so more row FFTs run at once.
+// Batch: warps of a fixed grid take row items (run, y0, rows) round robin.
+// Rows of up to 512 take the lane form of the single run, a few rows of one
+// run per item (the tables of a row length are set up once per item); it
+// needs a little more instructions per row than the wide form below, but an
+// item is a tenth as long, so that a batch of any size fills the GPU evenly.
+// Rows of 1024 and 2048 take the wide form, 2048 / Nx rows at once.
+// EMAX: the widest row shape of the batch (Nx / 64).
+template <int E, bool INV>
+__device__ __forceinline__ void batch_lane_rows(const PoissonArgs& a, int y0, int y1, float2* sm) {
+  const int lane = threadIdx.x & 31;
+  const float2* __restrict__ tw = static_cast<const float2*>(a.tw);
+  LaneFft<E> fft;
+  float2 wk[E];
+  fft.init(tw, lane);
+  if constexpr (INV) {
+#pragma unroll
+    for (int n2 = 0; n2 < E; ++n2) wk[n2] = cmf1(tw[lane], tw[32 * n2]);
+  } else {
+    untangle_factors<E>(tw, lane, wk);
+  }
+  for (int y = y0; y < y1; ++y) {
+    if constexpr (INV)
+      irfft_lane_row<E, false>(a, y, fft, wk, sm);
+    else
+      rfft_lane_row<E>(a, y, fft, wk, sm);
+    __syncwarp();  // the row buffer is free for the next row
+  }
+}
+
 template <bool INV, int EMAX>
 __device__ __forceinline__ void batch_fft_body(const BatchTables& t, int step) {
-  __shared__ float2 smem[4][32 * 33];
+  __shared__ float2 smem[4][EMAX <= 8 ? EMAX * 34 : 32 * 33];
   const int warp = threadIdx.x >> 5;
   const int n = t.counts[2];
-  int* counter = t.work + (INV ? 3 : 1);
-  for (int it = next_item_warp(counter); it < n; it = next_item_warp(counter)) {
+  float2* sm = smem[warp];
+  for (int it = blockIdx.x * 4 + warp; it < n; it += gridDim.x * 4) {
     const int2 w = t.row_items[it];
     const BatchRunDesc& rd = t.runs[w.x];
     if (step >= rd.remaining) continue;
-    const PoissonArgs a = rd.pa;
-    float2* sm = smem[warp];
+    const PoissonArgs& a = rd.pa;
+    const int y0 = row_item_row(w.y), y1 = min(y0 + row_item_count(w.y), a.Ny);
     switch (rd.E) {
-      case 1: INV ? irfft_warp_rows<1, 32>(a, w.y, sm) : rfft_warp_rows<1, 32>(a, w.y, sm); break;
+      case 1: batch_lane_rows<1, INV>(a, y0, y1, sm); break;
       case 2:
-        if constexpr (EMAX >= 2) INV ? irfft_warp_rows<2, 16>(a, w.y, sm) : rfft_warp_rows<2, 16>(a, w.y, sm);
+        if constexpr (EMAX >= 2) batch_lane_rows<2, INV>(a, y0, y1, sm);
         break;
       case 4:
-        if constexpr (EMAX >= 4) INV ? irfft_warp_rows<4, 8>(a, w.y, sm) : rfft_warp_rows<4, 8>(a, w.y, sm);
+        if constexpr (EMAX >= 4) batch_lane_rows<4, INV>(a, y0, y1, sm);
         break;
       case 8:
-        if constexpr (EMAX >= 8) INV ? irfft_warp_rows<8, 4>(a, w.y, sm) : rfft_warp_rows<8, 4>(a, w.y, sm);
+        if constexpr (EMAX >= 8) batch_lane_rows<8, INV>(a, y0, y1, sm);
         break;
       case 16:
-        if constexpr (EMAX >= 16) INV ? irfft_warp_rows<16, 2>(a, w.y, sm) : rfft_warp_rows<16, 2>(a, w.y, sm);
+        if constexpr (EMAX >= 16) INV ? irfft_warp_rows<16, 2>(a, y0, sm) : rfft_warp_rows<16, 2>(a, y0, sm);
         break;
       default:
-        if constexpr (EMAX >= 32) INV ? irfft_warp_rows<32, 1>(a, w.y, sm) : rfft_warp_rows<32, 1>(a, w.y, sm);
+        if constexpr (EMAX >= 32) INV ? irfft_warp_rows<32, 1>(a, y0, sm) : rfft_warp_rows<32, 1>(a, y0, sm);
         break;
     }
   }
 }
 
+// (five CTAs per SM up to rows of 512; more registers than that leave too few
+// warps to cover the loads of their rows)
 template <int EMAX>
-__global__ void __launch_bounds__(128) k_batch_rfft(BatchTables t, int step) {
+__global__ void __launch_bounds__(128, EMAX <= 8 ? 5 : 1) k_batch_rfft(BatchTables t, int step) {
   grid_dep_wait();  // programmatic dependent launch (t.pdl): the previous phase has ended
   grid_dep_launch();
+  if (blockIdx.x == 0 && threadIdx.x == 0) t.work[0] = 0;  // the march is over: its counter for the next step
   batch_fft_body<false, EMAX>(t, step);
 }
 
@@ -667,6 +694,7 @@ template <int EMAX>
 __global__ void __launch_bounds__(128) k_batch_irfft(BatchTables t, int step) {
   grid_dep_wait();  // programmatic dependent launch (t.pdl): the previous phase has ended
   grid_dep_launch();
+  if (blockIdx.x == 0 && threadIdx.x == 0) t.work[1] = 0;  // the solves are over: their counter for the next step
   batch_fft_body<true, EMAX>(t, step);
 }
 
@@ -674,6 +702,7 @@ template <int EMAX>
 __global__ void __launch_bounds__(128, 5) k_batch_irfft_narrow(BatchTables t, int step) {
   grid_dep_wait();  // programmatic dependent launch (t.pdl): the previous phase has ended
   grid_dep_launch();
+  if (blockIdx.x == 0 && threadIdx.x == 0) t.work[1] = 0;  // the solves are over: their counter for the next step
   batch_fft_body<true, EMAX>(t, step);
 }
 

@@ -910,7 +910,9 @@ __global__ void __launch_bounds__(128, 3) k_batch_march(BatchTables t, int step)
   constexpr int NST = 2;
   unsigned char* ring = march_smem + (size_t)(threadIdx.x >> 5) * March2Stages<float, float, NST>::kBytesPerWarp;
   const int n = t.counts[1];
-  for (int it = next_item_warp(t.work); it < n; it = next_item_warp(t.work)) {
+  // the first item by position (a counter's answer is an L2 round trip)
+  const int nwarps = gridDim.x * 4;
+  for (int it = blockIdx.x * 4 + (threadIdx.x >> 5); it < n; it = nwarps + next_item_warp(t.work)) {
     const int4 w = t.march_items[it];
     const BatchRunDesc& rd = t.runs[w.x];
     if (step >= rd.remaining) continue;  // whole warp

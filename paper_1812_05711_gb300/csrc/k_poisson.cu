@@ -768,20 +768,25 @@ __global__ void __launch_bounds__(kTileThreads) k_batch_modes(BatchTables t, int
   grid_dep_wait();  // programmatic dependent launch (t.pdl): the forward transforms have ended
   grid_dep_launch();
   __shared__ TileScratch<float, kBatchTileModes, kTileThreads> ts;
+  __shared__ MeanScratch<float, kMeanThreadsSmall> ms;
   __shared__ int s_it;
-  const int n = t.counts[3];
-  for (;;) {
-    // the CTA takes the next tile (tallest runs first) from the step's counter
-    if (threadIdx.x == 0) s_it = atomicAdd(t.work + 2, 1);
-    __syncthreads();
-    const int it = s_it;
-    __syncthreads();
-    if (it >= n) break;
-    const int2 w = t.tile_items[it];
+  const int nmean = t.mean_in_modes ? t.counts[0] : 0, n = nmean + t.counts[3];
+  // the CTA's first item by its position, then the next one from the step's
+  // counter: the runs' mean modes (the longest chains), then the tiles,
+  // tallest runs first
+  for (int it = blockIdx.x; it < n;) {
+    const int2 w = it < nmean ? make_int2(it, -1) : t.tile_items[it - nmean];
     const BatchRunDesc& rd = t.runs[w.x];
-    if (step >= rd.remaining) continue;  // whole CTA
-    const PoissonArgs a = rd.pa;
-    modes_tile_body<float, kBatchTileModes, kTileThreads>(a, w.y, smem_raw, ts);
+    if (step < rd.remaining) {  // whole CTA
+      const PoissonArgs a = rd.pa;
+      if (w.y >= 0)
+        modes_tile_body<float, kBatchTileModes, kTileThreads>(a, w.y, smem_raw, ts);
+      else if (threadIdx.x < kMeanThreadsSmall)
+        mean_mode_body<float, kMeanThreadsSmall>(a, smem_raw, ms);
+    }
+    if (threadIdx.x == 0) s_it = (int)gridDim.x + atomicAdd(t.work + 1, 1);
+    __syncthreads();
+    it = s_it;
     __syncthreads();
   }
 }
