@@ -25,8 +25,10 @@
 
 #include <mutex>
 
+#include "cluster_dev.cuh"
 #include "ehd.h"
-#include "ehd_dev.cuh"
+#include "fft_dev.cuh"
+#include "mean_dev.cuh"
 
 namespace ehd {
 void set_error(const char* msg);
@@ -67,6 +69,9 @@ struct DeviceSlot {
   unsigned char* base = nullptr;  // device address of g_scratch at the last call
   int Nx = 0, Ny = 0, wall_mode = -1;  // sizes the tables were built for
   bool always_rebuild = false;    // set once a call was made during stream capture
+  // the cluster kernel of 64, 128, 256, 512 columns: most shared memory known
+  // to fit, least known not to
+  size_t fits[4] = {0, 0, 0, 0}, too_big[4] = {~size_t(0), ~size_t(0), ~size_t(0), ~size_t(0)};
 };
 std::mutex g_mu;
 DeviceSlot g_slots[kMaxDevices];
@@ -288,6 +293,240 @@ __global__ void __launch_bounds__(256) k_na_inv(int Nx, int Ny, float* __restric
     phi[(size_t)y * Nx + x] = (float)(pb + (double)(res[x].re / (float)Nx));
 }
 
+// ---------------------------------------------------------------- one launch
+// The whole solve by one cluster of 16 CTAs, for grids whose spectrum fits
+// their shared memory (64 to 512 columns, up to 2^18 nodes).  A small solve is
+// bound by its launches and by the chain of each kernel, not by the work: the
+// three kernels above take 26.6 us a call at 256 x 208 (radix-2 rows with a
+// barrier a stage, an FP64 elimination of the mean mode), of which the data
+// would take 0.1; this one takes 12.3 (64 x 56: 17.7 -> 7.4; 512 x 416: 32.8 ->
+// 26.6, the last size where 16 SMs are enough).  Here a warp transforms a row (LaneFft), the wavenumbers'
+// columns are written into the CTA that solves them and back into the rows'
+// owners, and the mean mode is the FP64 double prefix sum of the run's solver.
+namespace na {
+using namespace ehd;
+constexpr int kThreads = 512, kWarps = kThreads / 32;
+constexpr int kMeanCta = 8, kMeanWarp = kWarps - 4;  // the mean mode's CTA and its first warp there
+constexpr int kMeanNT = 128;
+
+template <int E>
+struct Lay {
+  static constexpr int Nx = 64 * E, L = 32 * E, kModes = L / kClusterCtas;
+  int rows, spec, col, row, mean, pb;  // float2 offsets
+  size_t bytes;
+  __host__ __device__ explicit Lay(int Ny) {
+    rows = (Ny + kClusterCtas - 1) / kClusterCtas;
+    spec = 0;
+    col = spec + rows * (L + 2);
+    row = col + kModes * (Ny + 1);
+    mean = row + kWarps * kLaneRow<E>;
+    pb = mean + 2 * Ny;
+    bytes = sizeof(float2) * (size_t)(pb + rows);
+  }
+};
+
+template <int E>
+__global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, float ieps, const float* __restrict__ rhoc,
+                                                       float* __restrict__ phi, Ptrs p, PoissonArgs pa) {
+  using La = Lay<E>;
+  constexpr int Nx = La::Nx, L = La::L, ML = La::kModes;
+  extern __shared__ __align__(16) float2 sm[];
+  __shared__ MeanScratch<double, kMeanNT> ms;
+  const La la(Ny);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int rank;
+  asm("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(rank));
+  const int r0 = band_start(rank, Ny), nr = band_start(rank + 1, Ny) - r0;
+  float2* const spec = sm + la.spec;
+  float2* const col = sm + la.col;
+  float2* const rowbuf = sm + la.row + warp * kLaneRow<E>;
+  double* const mean_v = reinterpret_cast<double*>(sm + la.mean);
+  double* const pb = reinterpret_cast<double*>(sm + la.pb);
+
+  const float2* __restrict__ tw = reinterpret_cast<const float2*>(p.tw);  // W_Nx^k, k < Nx / 2
+  auto W = [&](int k) {
+    const float2 v = tw[k & (Nx / 2 - 1)];
+    return (k & (Nx / 2)) ? make_float2(-v.x, -v.y) : v;
+  };
+  LaneFft<E, true> fft;
+#pragma unroll
+  for (int k2 = 0; k2 < E; ++k2) fft.w[k2] = W((2 * lane * k2) & (Nx - 1));
+  fft.init_stages(lane);
+  float2 wk[E];  // W_Nx^(lane + 32 j)
+#pragma unroll
+  for (int j = 0; j < E; ++j) wk[j] = tw[lane + 32 * j];
+  cluster_sync();  // every CTA runs: its shared memory may be written
+
+  // ---- rows: s = -rho_c / eps, its sum (pairs of FP32 numbers, exact), the
+  // transform of what differs from the row's first value
+  for (int r = warp; r < nr; r += kWarps) {
+    const int y = r0 + r;
+    const float2* src = reinterpret_cast<const float2*>(rhoc + (size_t)y * Nx);
+    float re[E], im[E];
+    float hi = 0.0f, lo = 0.0f;
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+      const float2 v = src[lane + 32 * j];
+      re[j] = -v.x * ieps;
+      im[j] = -v.y * ieps;
+    }
+    const float c0 = __shfl_sync(0xffffffffu, re[0], 0);
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+      float e;
+      two_sum_f(hi, re[j], hi, e);
+      lo += e;
+      two_sum_f(hi, im[j], hi, e);
+      lo += e;
+      re[j] -= c0;
+      im[j] -= c0;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      float e;
+      const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+      two_sum_f(hi, h2, hi, e);
+      lo = lo + l2 + e;
+    }
+    fft.run(re, im, lane);
+    if (lane == 0) {
+      st_peer(peer_addr(mean_v + y, kMeanCta), make_float2(hi, lo));
+      st_peer(peer_addr(col + (ML - 1) * (Ny + 1) + y, kClusterCtas - 1), make_float2(2.0f * (re[0] - im[0]), 0.0f));
+    }
+    lane_fft_store<E>(re, im, rowbuf, lane);
+    // S[k] = E + W^k O from E = Z[k] + Z*[L - k], O = (Z[k] - Z*[L - k]) / i
+    // (twice the coefficients: the halves join the inverse's scale)
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+      const int k = lane + 32 * j;
+      const float2 zk = rowbuf[lpad(k)], zp = rowbuf[lpad((L - k) & (L - 1))];
+      const float Er = zk.x + zp.x, Ei = zk.y - zp.y, Dr = zk.x - zp.x, Di = zk.y + zp.y;
+      const int m = k - 1;
+      if (m >= 0)
+        st_peer(peer_addr(col + (m % ML) * (Ny + 1) + y, m / ML),
+                make_float2(fmaf(wk[j].x, Di, fmaf(wk[j].y, Dr, Er)), fmaf(wk[j].y, Di, fmaf(-wk[j].x, Dr, Ei))));
+    }
+    __syncwarp();
+  }
+  cluster_sync();
+
+  // ---- y solves: a warp per wavenumber, 32 chunks of rows
+  const bool mean_warp = rank == kMeanCta && warp >= kMeanWarp;
+  if (mean_warp) {
+    const int t = tid - 32 * kMeanWarp;
+    for (int j = t; j < Ny; j += kMeanNT) {
+      const float2 v = reinterpret_cast<const float2*>(mean_v)[j];
+      mean_v[j] = (double)v.x + (double)v.y;
+    }
+    sub_sync<kMeanNT>();
+    mean_mode_core<double, kMeanNT>(pa, mean_v, ms, t, [&](int j, double pc, double) {
+      const int o = band_owner(j, Ny);
+      const unsigned long long b = __double_as_longlong(pc);
+      st_peer(peer_addr(pb + (j - band_start(o, Ny)), o),
+              make_float2(__uint_as_float((unsigned)b), __uint_as_float((unsigned)(b >> 32))));
+    });
+  } else {
+    const int nw = rank == kMeanCta ? kMeanWarp : kWarps;
+    const int C = (Ny + 31) >> 5, j0 = min(lane * C, Ny), j1 = min(j0 + C, Ny);
+    for (int q = warp; q < ML; q += nw) {
+      const int m = rank * ML + q + 1;
+      const float* __restrict__ r = p.piv + (size_t)m * Ny;
+      float2* d = col + q * (Ny + 1);
+      float al = 1.0f;
+      float2 br = make_float2(0.0f, 0.0f);
+      for (int j = j0; j < j1; ++j) {
+        const float rj = r[j];
+        const float2 v = d[j];
+        al = -rj * al;
+        br = make_float2(rj * (v.x - br.x), rj * (v.y - br.y));
+      }
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const float a2 = __shfl_up_sync(0xffffffffu, al, o);
+        const float bx = __shfl_up_sync(0xffffffffu, br.x, o), by = __shfl_up_sync(0xffffffffu, br.y, o);
+        if (lane >= o) {
+          br = make_float2(fmaf(al, bx, br.x), fmaf(al, by, br.y));
+          al *= a2;
+        }
+      }
+      float2 x = make_float2(__shfl_up_sync(0xffffffffu, br.x, 1), __shfl_up_sync(0xffffffffu, br.y, 1));
+      if (lane == 0) x = make_float2(0.0f, 0.0f);
+      al = 1.0f;
+      br = make_float2(0.0f, 0.0f);
+      for (int j = j0; j < j1; ++j) {
+        const float rj = r[j];
+        const float2 v = d[j];
+        x = make_float2(rj * (v.x - x.x), rj * (v.y - x.y));
+        d[j] = x;
+        br = make_float2(fmaf(al, x.x, br.x), fmaf(al, x.y, br.y));
+        al = -al * rj;
+      }
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const float a2 = __shfl_down_sync(0xffffffffu, al, o);
+        const float bx = __shfl_down_sync(0xffffffffu, br.x, o), by = __shfl_down_sync(0xffffffffu, br.y, o);
+        if (lane + o < 32) {
+          br = make_float2(fmaf(al, bx, br.x), fmaf(al, by, br.y));
+          al *= a2;
+        }
+      }
+      x = make_float2(__shfl_down_sync(0xffffffffu, br.x, 1), __shfl_down_sync(0xffffffffu, br.y, 1));
+      if (lane == 31) x = make_float2(0.0f, 0.0f);
+      int o = j1 > j0 ? band_owner(j1 - 1, Ny) : 0, b0 = band_start(o, Ny);
+      for (int j = j1 - 1; j >= j0; --j) {
+        const float2 v = d[j];
+        x = make_float2(fmaf(-r[j], x.x, v.x), fmaf(-r[j], x.y, v.y));
+        if (j < b0) b0 = band_start(--o, Ny);  // (every band has a row)
+        st_peer(peer_addr(spec + (j - b0) * (L + 2) + m, o), x);
+      }
+    }
+  }
+  cluster_sync();
+
+  // ---- rows back: phi = mean + inverse transform, the sum in pairs
+  const float scale = 0.25f / (float)L;  // both halves and 1 / L
+  for (int r = warp; r < nr; r += kWarps) {
+    const float2* s = spec + r * (L + 2);
+    float re[E], im[E];
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+      const int k = lane + 32 * j;
+      const float2 sk = (k == 0) ? make_float2(0.0f, 0.0f) : s[k], sp = s[L - k];
+      const float Er = sk.x + sp.x, Ei = sk.y - sp.y, Dr = sk.x - sp.x, Di = sk.y + sp.y;
+      const float Or = fmaf(Dr, wk[j].x, Di * wk[j].y), Oi = fmaf(Di, wk[j].x, -Dr * wk[j].y);
+      re[j] = Er - Oi;
+      im[j] = -(Ei + Or);
+    }
+    fft.run(re, im, lane);
+    lane_fft_store<E>(re, im, rowbuf, lane);
+    const ff b = ff_from(pb[r]);
+    float2* out = reinterpret_cast<float2*>(phi + (size_t)(r0 + r) * Nx);
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+      const float2 v = rowbuf[lpad(lane + 32 * j)];
+      float hx, ex, hy, ey;
+      two_sum_f(b.hi, v.x * scale, hx, ex);
+      two_sum_f(b.hi, -v.y * scale, hy, ey);
+      out[lane + 32 * j] = make_float2(hx + (ex + b.lo), hy + (ey + b.lo));
+    }
+    __syncwarp();
+  }
+}
+
+// The cluster kernel of a grid, nullptr where it does not apply.
+using Kernel = void (*)(int, float, const float*, float*, Ptrs, PoissonArgs);
+Kernel pick(int Nx, int Ny, size_t* smem) {
+  if (Ny < kClusterCtas || (long long)Nx * Ny > (1LL << 18)) return nullptr;
+  switch (Nx) {
+    case 64: *smem = Lay<1>(Ny).bytes; return k_solve<1>;
+    case 128: *smem = Lay<2>(Ny).bytes; return k_solve<2>;
+    case 256: *smem = Lay<4>(Ny).bytes; return k_solve<4>;
+    case 512: *smem = Lay<8>(Ny).bytes; return k_solve<8>;
+  }
+  return nullptr;
+}
+}  // namespace na
+
 ehd_status na_fail(ehd_status st, const char* msg) {
   ehd::set_error(msg);
   return st;
@@ -338,6 +577,32 @@ extern "C" ehd_status ehd_poisson_noalloc(int Nx, int Ny, double eps, double phi
     slot.Nx = Nx;
     slot.Ny = Ny;
     slot.wall_mode = wall_mode;
+  }
+  size_t smem = 0;
+  na::Kernel kernel = na::pick(Nx, Ny, &smem);
+  // rows are read and written as pairs
+  if (kernel && ((reinterpret_cast<uintptr_t>(rhoc) | reinterpret_cast<uintptr_t>(phi)) & 7) == 0) {
+    const int i = Nx == 64 ? 0 : Nx == 128 ? 1 : Nx == 256 ? 2 : 3;
+    if (smem > slot.fits[i] && smem < slot.too_big[i]) {
+      if (ehd::cluster_fits(kernel, na::kThreads, smem))
+        slot.fits[i] = smem;
+      else
+        slot.too_big[i] = smem;
+    }
+    if (smem <= slot.fits[i]) {
+      ehd::PoissonArgs pa{};
+      pa.Nx = Nx;
+      pa.Ny = Ny;
+      pa.wall_mode = wall_mode;
+      pa.mW = (double)Nx * phi0;
+      pa.mC = (wall_mode == 0) ? 1.0 / (2.0 * Ny) : 1.0 / (double)(Ny + 1);
+      cudaLaunchAttribute at[1];
+      cudaLaunchConfig_t c;
+      ehd::cluster_launch_config(&c, at, na::kThreads, smem, s);
+      if (cudaLaunchKernelEx(&c, kernel, Ny, (float)(1.0 / eps), rhoc, phi, p, pa) != cudaSuccess)
+        return na_fail(EHD_ECUDA, "ehd_poisson_noalloc: kernel launch failed");
+      return EHD_OK;
+    }
   }
   const size_t row_smem = 2 * (size_t)Nx * sizeof(Cplx<float>);
   k_na_fwd<<<Ny, 256, row_smem, s>>>(Nx, Ny, 1.0 / eps, rhoc, p);

@@ -139,7 +139,43 @@ __device__ __forceinline__ float2 cmf0(float2 a, float2 b) {
 __device__ __forceinline__ float2 cmf1(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -(a.y * b.y)), fmaf(a.y, b.x, a.x * b.y));
 }
+// LIT: the E-point transform by literal factors (fft_lit), for a unit that does
+// not set the tables and owes nobody its bits.
 template <int E>
+__device__ __forceinline__ void fft_lit(float (&re)[E], float (&im)[E]) {
+  if constexpr (E == 2) {
+    const float r = re[0], i = im[0];
+    re[0] = r + re[1];
+    im[0] = i + im[1];
+    re[1] = r - re[1];
+    im[1] = i - im[1];
+  } else if constexpr (E > 2) {  // even and odd halves, then W_E^k
+    float er[E / 2], ei[E / 2], orr[E / 2], oi[E / 2];
+#pragma unroll
+    for (int k = 0; k < E / 2; ++k) {
+      er[k] = re[2 * k];
+      ei[k] = im[2 * k];
+      orr[k] = re[2 * k + 1];
+      oi[k] = im[2 * k + 1];
+    }
+    fft_lit<E / 2>(er, ei);
+    fft_lit<E / 2>(orr, oi);
+    constexpr float h = 0.70710678118654752440f;
+#pragma unroll
+    for (int k = 0; k < E / 2; ++k) {
+      // W_E^k for E = 4 and 8: k (8 / E) eighths of a turn
+      const int q = k * (8 / E);
+      const float c = q == 0 ? 1.0f : (q == 1 ? h : (q == 2 ? 0.0f : -h));
+      const float s = q == 0 ? 0.0f : (q == 2 ? -1.0f : -h);
+      const float tr = orr[k] * c - oi[k] * s, ti = orr[k] * s + oi[k] * c;
+      re[k] = er[k] + tr;
+      im[k] = ei[k] + ti;
+      re[k + E / 2] = er[k] - tr;
+      im[k + E / 2] = ei[k] - ti;
+    }
+  }
+}
+template <int E, bool LIT = false>
 struct LaneFft {
   float2 w[E];   // W_L^(lane k2)
   float2 ws[5];  // this lane's butterfly factor in each stage
@@ -150,6 +186,9 @@ struct LaneFft {
 #pragma unroll
     for (int k2 = 1; k2 < E; ++k2)
       w[k2] = k2 == 1 ? base : ((k2 & 3) == 0) ? tw[(2 * lane * k2) & (64 * E - 1)] : cmf0(w[k2 - 1], base);
+    init_stages(lane);
+  }
+  __device__ __forceinline__ void init_stages(int lane) {
     const int p = __brev((unsigned)lane) >> 27;
 #pragma unroll
     for (int s = 0; s < 5; ++s) {
@@ -158,7 +197,10 @@ struct LaneFft {
     }
   }
   __device__ __forceinline__ void run(float (&re)[E], float (&im)[E], int lane) const {
-    fft_reg<E>(re, im);
+    if constexpr (LIT)
+      fft_lit<E>(re, im);
+    else
+      fft_reg<E>(re, im);
 #pragma unroll
     for (int k2 = 0; k2 < E; ++k2) {
       const float2 v = cmf1(make_float2(re[k2], im[k2]), w[k2]);

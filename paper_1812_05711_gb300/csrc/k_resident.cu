@@ -29,6 +29,7 @@
 // two copies of the populations (36 floats a node) must fit beside the rest;
 // a cluster spans at most one GPC.  Larger runs keep the multi-kernel step,
 // which has all SMs.
+#include "cluster_dev.cuh"
 #include "fft_dev.cuh"
 #include "march_dev.cuh"
 #include "mean_dev.cuh"
@@ -37,37 +38,13 @@ namespace ehd {
 
 namespace {
 
-constexpr int kCtas = 16;
 constexpr int kThreads = 512;
 constexpr int kRowWarps = 8;    // a CTA owns at most 8 rows
-constexpr int kMaxRows = kCtas * kRowWarps;
+constexpr int kMaxRows = kClusterCtas * kRowWarps;
 constexpr int kChunkRows = 4;   // rows per lane in the wavenumber solve (Ny <= 128)
 constexpr int kMeanCta = 8;     // neither wall's CTA
 constexpr int kMeanWarp = 8;    // its first warp of the mean mode (four of them)
 constexpr int kFluxWarp = 8;    // first flux warp of the wall CTAs, one per 60-column strip
-
-__device__ __forceinline__ void cluster_arrive() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void cluster_sync() {
-  __syncwarp();
-  cluster_arrive();
-  cluster_wait();
-}
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-// the address of p's counterpart in CTA `rank` of the cluster
-__device__ __forceinline__ unsigned peer_addr(const void* p, int rank) {
-  unsigned r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void st_peer(unsigned a, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(a), "f"(v) : "memory");
-}
-__device__ __forceinline__ void st_peer(unsigned a, float2 v) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};\n" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
-}
 
 // four populations of the storage type, as floats (see Store)
 template <class S>
@@ -104,15 +81,11 @@ struct Four<__half> {
   }
 };
 
-// first row of CTA c's band, and the CTA that owns row j
-__host__ __device__ __forceinline__ int band_start(int c, int Ny) { return c * Ny / kCtas; }
-__device__ __forceinline__ int band_owner(int j, int Ny) { return ((j + 1) * kCtas - 1) / Ny; }
-
 // Shared memory of a CTA (floats from its start), RM rows at most per band.
 template <int E>
 struct Layout {
   static constexpr int Nx = 64 * E, L = 32 * E;
-  static constexpr int kModes = L / kCtas;  // wavenumbers per CTA: m = rank kModes + 1 ...
+  static constexpr int kModes = L / kClusterCtas;  // wavenumbers per CTA: m = rank kModes + 1 ...
   static constexpr int kSpecRow = 2 * (L + 2);
   static constexpr int kStrips = (Nx + 59) / 60;
   int pop, phi, spec, col, col_row, row, mean, ebar, shift, flux, total;
@@ -200,9 +173,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(StepArgs a, PoissonArg
     const int m = lane + 32 * q - 1;
     to_col[q] = (m >= 0 && warp < nr) ? peer_addr(col + (m % ML) * (lay.col_row / 2) + myrow, m / ML) : 0u;
   }
-  if (warp < nr) to_nyq = peer_addr(col + (ML - 1) * (lay.col_row / 2) + myrow, kCtas - 1);
+  if (warp < nr) to_nyq = peer_addr(col + (ML - 1) * (lay.col_row / 2) + myrow, kClusterCtas - 1);
   const unsigned to_mean = warp < nr ? peer_addr(mean_v + myrow, kMeanCta) : 0u;
-  const bool wall_lo = rank == 0, wall_hi = rank == kCtas - 1;
+  const bool wall_lo = rank == 0, wall_hi = rank == kClusterCtas - 1;
   const int strip = warp - kFluxWarp;
   const bool flux_warp = (wall_lo || wall_hi) && strip >= 0 && strip < Lay::kStrips;
   double flux_total = (flux_warp && strip == 0) ? pa.flux_acc[wall_hi ? 1 : 0] : 0.0;
@@ -557,7 +530,7 @@ namespace {
 
 using ResidentKernel = void (*)(StepArgs, PoissonArgs, int, int);
 
-int max_rows(int Ny) { return (Ny + kCtas - 1) / kCtas; }
+int max_rows(int Ny) { return (Ny + kClusterCtas - 1) / kClusterCtas; }
 
 template <int E>
 bool resident_config_n(int storage, int Ny, ResidentKernel* k, size_t* smem) {
@@ -570,27 +543,13 @@ bool resident_config_n(int storage, int Ny, ResidentKernel* k, size_t* smem) {
   return false;
 }
 bool resident_config(int Nx, int Ny, int storage, ResidentKernel* k, size_t* smem) {
-  if (Ny < kCtas || Ny > kMaxRows) return false;
+  if (Ny < kClusterCtas || Ny > kMaxRows) return false;
   switch (Nx) {
     case 64: return resident_config_n<1>(storage, Ny, k, smem);
     case 128: return resident_config_n<2>(storage, Ny, k, smem);
     case 256: return resident_config_n<4>(storage, Ny, k, smem);
   }
   return false;
-}
-
-void resident_launch_config(cudaLaunchConfig_t* c, cudaLaunchAttribute* at, size_t smem, cudaStream_t s) {
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = kCtas;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  *c = cudaLaunchConfig_t{};
-  c->gridDim = dim3(kCtas);
-  c->blockDim = dim3(kThreads);
-  c->dynamicSmemBytes = smem;
-  c->stream = s;
-  c->attrs = at;
-  c->numAttrs = 1;
 }
 
 }  // namespace
@@ -601,21 +560,7 @@ bool resident_supported(int Nx, int Ny, int storage) {
   ResidentKernel k = nullptr;
   size_t smem = 0;
   if (!resident_config(Nx, Ny, storage, &k, &smem)) return false;
-  int dev = 0, optin = 0, n = 0;
-  cudaFuncAttributes fa;
-  cudaLaunchAttribute at[1];
-  cudaLaunchConfig_t c;
-  resident_launch_config(&c, at, smem, nullptr);
-  const bool ok = cudaGetDevice(&dev) == cudaSuccess &&
-                  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
-                  cudaFuncGetAttributes(&fa, k) == cudaSuccess && smem + fa.sharedSizeBytes <= (size_t)optin &&
-                  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       optin - (int)fa.sharedSizeBytes) == cudaSuccess &&
-                  cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                  cudaOccupancyMaxActiveClusters(&n, k, &c) == cudaSuccess && n >= 1 &&
-                  fft_set_tables() == cudaSuccess;
-  if (!ok) (void)cudaGetLastError();
-  return ok;
+  return cluster_fits(k, kThreads, smem) && fft_set_tables() == cudaSuccess;
 }
 
 cudaError_t launch_resident(const StepArgs& a, const PoissonArgs& pa, int storage, int steps, cudaStream_t s) {
@@ -624,7 +569,7 @@ cudaError_t launch_resident(const StepArgs& a, const PoissonArgs& pa, int storag
   if (!resident_config(a.Nx, a.Ny, storage, &k, &smem)) return cudaErrorInvalidValue;
   cudaLaunchAttribute at[1];
   cudaLaunchConfig_t c;
-  resident_launch_config(&c, at, smem, s);
+  cluster_launch_config(&c, at, kThreads, smem, s);
   return cudaLaunchKernelEx(&c, k, a, pa, steps, max_rows(a.Ny));
 }
 
