@@ -140,8 +140,8 @@ struct ehd_run {
   double* bsum = nullptr;  // [4][Ny] rho_c, rho, j_y, j_x of the newest base state, [2][Ny] + [2][chunks] its prefix sums
   double* bmom = nullptr;  // [5][Ny] its moments for the next base step
   float* btab[2] = {nullptr, nullptr};
-  cudaStream_t side2 = nullptr;  // the base chain: forked after the march, joined at the end of the step
-  cudaEvent_t ev_base = nullptr;
+  cudaStream_t side2 = nullptr;  // the base chain: forked at the start of the step, joined at its end
+  cudaEvent_t ev_base = nullptr, ev_start = nullptr;
 };
 
 struct ehd_batch {
@@ -151,7 +151,7 @@ struct ehd_batch {
   std::vector<size_t> member_bytes;
   cudaStream_t stream = nullptr, side = nullptr;
   bool own_stream = false;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_upload = nullptr, ev_base = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_upload = nullptr, ev_base = nullptr, ev_start = nullptr;
   cudaStream_t side2 = nullptr;  // base chains of perturbation-form members
   std::vector<ehd_run*> members;
   int npert = 0;              // members in the perturbation form
@@ -395,14 +395,15 @@ BaseArgs base_step_args(const ehd_run* r, int cur) {
   return b;
 }
 // The base step from buffer `cur` and the potential and march table of the
-// result, on the third stream from the point where the departure's forward
-// row transform has ended (ev_fork: the base kernels then run beside the
-// wavenumber solves and the inverse transform rather than holding SM slots
-// the march or the forward transform need: 125.3 us per 2048 x 1680 step
-// against 127.7 when forked right after the march, and 122.4 for the shifted
-// FP32 form); the main stream waits for them at the end of the step.
+// result, on the third stream; the main stream waits for them at the end of
+// the step.  The base depends on nothing of the departure's step, so it starts
+// with it (fork_base, before the march) and runs beside all of it: the chain
+// of FP64 instructions is as long as a small run's whole step (128 x 104: 15.1
+// us per step against 25.8 when forked after the forward row transform,
+// 512 x 416: 20.1 / 29.0, 2048 x 1680: 115.5 / 120.5).
+cudaError_t fork_base(ehd_run* r) { return r->pert ? cudaEventRecord(r->ev_start, r->stream) : cudaSuccess; }
 cudaError_t enqueue_base(ehd_run* r, int cur) {
-  cudaError_t e = cudaStreamWaitEvent(r->side2, r->ev_fork, 0);
+  cudaError_t e = cudaStreamWaitEvent(r->side2, r->ev_start, 0);
   if (e == cudaSuccess) e = launch_base_step(base_step_args(r, cur), r->side2);
   if (e == cudaSuccess) e = launch_base_poisson(base_poisson_args(r, 1 - cur), r->side2);
   if (e == cudaSuccess) e = cudaEventRecord(r->ev_base, r->side2);
@@ -483,7 +484,8 @@ cudaError_t enqueue_step(ehd_run* r, int cur, long k) {
     sa.slab_off = march_shift(r, k);
     PoissonArgs pa = poisson_args(r, true);
     pa.xoff = sa.slab_off;
-    cudaError_t e = launch_march_run(r, sa, cur);
+    cudaError_t e = fork_base(r);
+    if (e == cudaSuccess) e = launch_march_run(r, sa, cur);
     if (e == cudaSuccess) e = launch_poisson(pa, r->real_f64, r->stream, r->side, r->ev_fork, r->ev_join);
     if (e == cudaSuccess && r->pert) e = enqueue_base(r, cur);
     if (e == cudaSuccess && r->pert) e = cudaStreamWaitEvent(r->stream, r->ev_base, 0);
@@ -554,6 +556,7 @@ ehd_status destroy_quiet(ehd_run* r) {
   if (r->ev_fork) cudaEventDestroy(r->ev_fork);
   if (r->ev_join) cudaEventDestroy(r->ev_join);
   if (r->ev_base) cudaEventDestroy(r->ev_base);
+  if (r->ev_start) cudaEventDestroy(r->ev_start);
   if (r->side) cudaStreamDestroy(r->side);
   if (r->side2) cudaStreamDestroy(r->side2);
   std::vector<void*> bl = r->blocks;
@@ -724,7 +727,8 @@ ehd_status ehd_create(int Nx, int Ny, double T, double C, double M, double Fe, d
       cudaEventCreateWithFlags(&r->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&r->ev_join, cudaEventDisableTiming) != cudaSuccess ||
       (o.perturbation && (cudaStreamCreateWithFlags(&r->side2, cudaStreamNonBlocking) != cudaSuccess ||
-                          cudaEventCreateWithFlags(&r->ev_base, cudaEventDisableTiming) != cudaSuccess))) {
+                          cudaEventCreateWithFlags(&r->ev_base, cudaEventDisableTiming) != cudaSuccess ||
+                          cudaEventCreateWithFlags(&r->ev_start, cudaEventDisableTiming) != cudaSuccess))) {
     destroy_quiet(r);
     return fail(EHD_ECUDA, "stream/event creation failed");
   }
@@ -780,20 +784,22 @@ ehd_status ehd_create(int Nx, int Ny, double T, double C, double M, double Fe, d
   }
   r->step_kernel = (o.step_kernel >= 0) ? o.step_kernel : (r->real_f64 && !o.ex_spectral) ? 1 : 0;
   // programmatic dependent launch (mask of EHD_TUNE_PDL), as measured per
-  // step: all three Poisson kernels (7) for up to 2^18 nodes (512 x 416:
-  // 20.1 us against 20.7 with 3) and from 2^21 (2048 x 1680: 114.1 against
-  // 114.3 with 11, 114.7 with 3, 116.9 with none); between them the forward
-  // transform, the wavenumber solve and the step kernel (11; 1024 x 840: 41.2
-  // against 41.7 with 7, 42.4 with 3).  Perturbation-form runs take 11 at
-  // every size (512 x 416: 28.9 against 29.5 with 7; 2048 x 1680: 120.2
-  // against 121.1 with 3 and 135.4 with 7, whose early-resident inverse
-  // transform CTAs starve the base chain on the third stream)
+  // step.  Up to 2^18 nodes all four kernels (15; 256 x 205: 15.5 us against
+  // 15.9 with 7, 512 x 416 19.4 / 19.8; perturbation form 128 x 104 15.1 /
+  // 15.3); from 2^21 the three Poisson kernels (7; 2048 x 1680: 114.1 against
+  // 114.7 with 3, 116.9 with none); between them the forward transform, the
+  // wavenumber solve and the step kernel (11; 1024 x 840: 41.3 against 41.7
+  // with 7, 42.4 with 3), and so the larger perturbation-form runs (1024 x
+  // 840: 45.3 against 48.6 with 7)
   {
     const long long nodes = (long long)Nx * Ny;
     // FP64 runs: every kernel; none of them releases its successor early (see
     // k_modes64), so that all sizes gain or break even (16 x 100: 22.4 us
     // against 23.2 without; 128 x 104: 25.1 / 25.3; 1024 x 840: 317.3 / 317.3)
-    r->pdl = r->real_f64 ? 15 : (r->pert || (nodes > (1LL << 18) && nodes < (1LL << 21))) ? 11 : 7;
+    if (r->real_f64 || nodes <= (1LL << 18))
+      r->pdl = 15;
+    else
+      r->pdl = (r->pert || nodes < (1LL << 21)) ? 11 : 7;
   }
   r->cols_per_lane = 2;
   r->nstrips = march_strips(Nx, r->cols_per_lane);
@@ -1186,6 +1192,7 @@ ehd_status ehd_step_profile(ehd_run* r, long n, double* ms_out) {
     pa.xoff = sa.slab_off;
     const int nxt = 1 - r->cur;
     if (e == cudaSuccess) e = cudaEventRecord(E[0], r->stream);
+    if (e == cudaSuccess) e = fork_base(r);
     if (e == cudaSuccess)
       e = (r->step_kernel == 0) ? launch_march_run(r, sa, r->cur)
                                 : launch_step(sa, r->storage, r->real_f64, r->rows, r->stream);
@@ -1405,6 +1412,7 @@ void batch_free(ehd_batch* b) {
   if (b->ev_join) cudaEventDestroy(b->ev_join);
   if (b->ev_upload) cudaEventDestroy(b->ev_upload);
   if (b->ev_base) cudaEventDestroy(b->ev_base);
+  if (b->ev_start) cudaEventDestroy(b->ev_start);
   if (b->side2) cudaStreamDestroy(b->side2);
   if (b->side) cudaStreamDestroy(b->side);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
@@ -1481,21 +1489,22 @@ void batch_build_items(ehd_batch* b, int resident_warps) {
 
 // One tick of K steps.  With perturbation-form members (pert) each step
 // also advances their FP64 base states and base potentials on a third
-// stream, forked after the forward row transforms and joined at the end of
-// the step.
+// stream, forked at the start of the step (see enqueue_base) and joined at its
+// end.
 ehd_status batch_capture(ehd_batch* b, int K, bool pert, cudaGraphExec_t* out) {
   const BatchTables t = batch_tables(b);
   cudaGraph_t g = nullptr;
   EHD_CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
   for (int s = 0; s < K && e == cudaSuccess; ++s) {
-    e = launch_batch_march(t, s, b->grid_march, pert, b->stream);
+    if (pert) e = cudaEventRecord(b->ev_start, b->stream);
+    if (e == cudaSuccess) e = launch_batch_march(t, s, b->grid_march, pert, b->stream);
     if (e == cudaSuccess) e = launch_batch_rfft(t, s, b->grid_rows, b->stream);
     const bool side = !t.mean_in_modes;
-    if (e == cudaSuccess && (side || pert)) e = cudaEventRecord(b->ev_fork, b->stream);
+    if (e == cudaSuccess && side) e = cudaEventRecord(b->ev_fork, b->stream);
     if (e == cudaSuccess && side) e = cudaStreamWaitEvent(b->side, b->ev_fork, 0);
     if (pert) {
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side2, b->ev_fork, 0);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side2, b->ev_start, 0);
       if (e == cudaSuccess) e = launch_batch_base(t, s, b->max_runs, b->max_ny, b->side2);
       if (e == cudaSuccess) e = cudaEventRecord(b->ev_base, b->side2);
     }
@@ -1560,6 +1569,7 @@ ehd_status ehd_batch_create(int max_runs, size_t hbm_budget, int max_nx, int max
       cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&b->ev_upload, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&b->ev_base, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&b->ev_start, cudaEventDisableTiming) != cudaSuccess ||
       cudaStreamCreateWithFlags(&b->side2, cudaStreamNonBlocking) != cudaSuccess) {
     batch_free(b);
     return fail(EHD_ECUDA, "stream/event creation failed");
