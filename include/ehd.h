@@ -170,11 +170,12 @@ ehd_status ehd_step(ehd_run* run, long n);
  * no counterpart (measurement only).  host ms_out[EHD_NPROFILE]: summed
  * milliseconds of [0] the fused collide-stream kernel, [1] the charge-moment
  * kernel (0 when the step kernel writes the charge itself), [2] the Poisson
- * solve (forward FFT, tridiagonal modes, inverse FFT; the mean mode runs
- * beside them on a second stream and is joined before the event), [3] whole
+ * solve (forward FFT, tridiagonal modes, inverse FFT and the mean mode, in the
+ * launch of one of them or, for rows of 16, 32 and 2048 or more than 1024 rows
+ * in FP32, beside them on a second stream), [3] whole
  * steps, [4] = n, and inside [2]: [5] the forward row FFT, [6] the solves of
- * the wavenumbers m >= 1, [7] the inverse row FFT, [8] the mean mode m = 0
- * (on its own stream, concurrent with [6]).  Synchronises. */
+ * the wavenumbers m >= 1, [7] the inverse row FFT, [8] the launch that
+ * holds the mean mode m = 0.  Synchronises. */
 #define EHD_NPROFILE 9
 ehd_status ehd_step_profile(ehd_run* run, long n, double* ms_out);
 
@@ -191,10 +192,10 @@ ehd_status ehd_step_profile(ehd_run* run, long n, double* ms_out);
  * each is resident and waiting when its predecessor ends: 1 the forward row
  * transform, 2 the wavenumber solve, 4 the inverse transform, 8 the step
  * kernel (march form: it stages its first rows' populations before waiting
- * for phi); the default is 15 up to 2^18 nodes and for FP64 compute, 7 from
- * 2^21 nodes (2048 x 1680: 114.1 us per step against 114.7 with 3, 116.9 with
- * none), 11 between them (1024 x 840: 41.3 against 41.7 with 7) and for
- * larger perturbation-form runs; results are the same for every mask),
+ * for phi); the default is 15 up to 3 2^16 nodes and for FP64 compute, 4
+ * between 2^19 and 2^21 nodes (1024 x 840: 39.2 us per step against 41.2 with
+ * none) and 7 otherwise (2048 x 1680: 114.1 against 117.0 with none); results
+ * are the same for every mask),
  * EHD_TUNE_FFT_CTA (FP32 rows
  * of 2048: 1, the default, one CTA of 64 threads per row; 0, one warp per
  * row), EHD_TUNE_Y_SOLVER (the y solve of the wavenumbers m >= 1: 0, the

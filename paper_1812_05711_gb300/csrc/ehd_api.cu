@@ -784,22 +784,19 @@ ehd_status ehd_create(int Nx, int Ny, double T, double C, double M, double Fe, d
   }
   r->step_kernel = (o.step_kernel >= 0) ? o.step_kernel : (r->real_f64 && !o.ex_spectral) ? 1 : 0;
   // programmatic dependent launch (mask of EHD_TUNE_PDL), as measured per
-  // step.  Up to 2^18 nodes all four kernels (15; 256 x 205: 15.5 us against
-  // 15.9 with 7, 512 x 416 19.4 / 19.8; perturbation form 128 x 104 15.1 /
-  // 15.3); from 2^21 the three Poisson kernels (7; 2048 x 1680: 114.1 against
-  // 114.7 with 3, 116.9 with none); between them the forward transform, the
-  // wavenumber solve and the step kernel (11; 1024 x 840: 41.3 against 41.7
-  // with 7, 42.4 with 3), and so the larger perturbation-form runs (1024 x
-  // 840: 45.3 against 48.6 with 7)
+  // step.  FP64, and FP32 up to 3 2^16 nodes: all four kernels (15; 256 x 205:
+  // 13.7 us against 14.5 with 7 and 17.8 with none; 512 x 300: 19.0 / 19.2 /
+  // 21.5).  Up to 2^19 nodes the three Poisson kernels (7; 512 x 416: 19.6
+  // against 21.0 with 15), whose early CTAs no longer find room beside the
+  // march.  Up to 2^21 the inverse transform only, which carries the mean mode
+  // (4; 1024 x 840: 39.2 against 41.5 with 7, 41.2 with none).  Beyond, where
+  // the Poisson kernels are short against the march, all three again (7; 2048 x
+  // 1680: 114.1 against 114.7 with 6, 117.0 with none).  The perturbation form
+  // follows the same line (512 x 416: 20.3 with 7; 1024 x 840: 40.5 with 4,
+  // 44.2 with 7)
   {
     const long long nodes = (long long)Nx * Ny;
-    // FP64 runs: every kernel; none of them releases its successor early (see
-    // k_modes64), so that all sizes gain or break even (16 x 100: 22.4 us
-    // against 23.2 without; 128 x 104: 25.1 / 25.3; 1024 x 840: 317.3 / 317.3)
-    if (r->real_f64 || nodes <= (1LL << 18))
-      r->pdl = 15;
-    else
-      r->pdl = (r->pert || nodes < (1LL << 21)) ? 11 : 7;
+    r->pdl = (r->real_f64 || nodes <= (3LL << 16)) ? 15 : (nodes > (1LL << 19) && nodes < (1LL << 21)) ? 4 : 7;
   }
   r->cols_per_lane = 2;
   r->nstrips = march_strips(Nx, r->cols_per_lane);

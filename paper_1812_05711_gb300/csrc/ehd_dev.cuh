@@ -513,6 +513,9 @@ bool fftw_supported(int Nx);
 cudaError_t fftw_set_tables();
 cudaError_t launch_rfft_warp(const PoissonArgs& a, cudaStream_t s);
 cudaError_t launch_irfft_warp(const PoissonArgs& a, cudaStream_t s);
+// the inverse transform and, beside it and the wavenumber solve, the mean mode
+bool irfft_mean_supported(int Nx, int Ny);
+cudaError_t launch_irfft_mean(const PoissonArgs& a, cudaStream_t s);
 // The same transform of -i k_m phi_m (spectral E_x) into a.ex.
 cudaError_t launch_irfft_warp_dx(const PoissonArgs& a, cudaStream_t s);
 cudaError_t launch_fields(const FieldArgs& a, int storage, bool real_f64, unsigned mask, double* out,

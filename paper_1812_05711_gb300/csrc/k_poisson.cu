@@ -1332,32 +1332,42 @@ cudaError_t poisson_t(const PoissonArgs& a, cudaStream_t s, cudaStream_t side, c
   // solve, [2] after the inverse FFT (all on s); [3], [4] around the mean mode
   auto mark = [&](int k, cudaStream_t st) { return marks ? cudaEventRecord(marks[k], st) : cudaSuccess; };
   if ((e = mark(0, s)) != cudaSuccess) return e;
-  if (sizeof(R) == 8 && a.y_solver != 1) {
+  // where the mean mode runs: FP64, in the launch of the wavenumber solves;
+  // FP32, in the inverse transform's, where rows and their number allow; else
+  // on the second stream
+  const bool modes64 = sizeof(R) == 8 && a.y_solver != 1;
+  const bool with_inverse = warp_fft && irfft_mean_supported(a.Nx, a.Ny);
+  if (modes64 || with_inverse) side = nullptr;
+  if (modes64) {
     if ((e = mark(3, s)) != cudaSuccess) return e;
     if ((e = launch_modes64(a, s)) != cudaSuccess) return e;
     if ((e = mark(4, s)) != cudaSuccess) return e;
-    side = nullptr;
   } else {
     if (side) {
       if ((e = cudaEventRecord(fork, s)) != cudaSuccess) return e;
       if ((e = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess) return e;
     }
-    const cudaStream_t ms = side ? side : s;
-    if ((e = mark(3, ms)) != cudaSuccess) return e;
-    const size_t msm = 2 * (size_t)a.Ny * sizeof(typename MeanNum<R>::T);
-    if (a.Ny <= kMeanSmallRows)
-      k_mean_mode<R, kMeanThreadsSmall><<<1, kMeanThreadsSmall, msm, ms>>>(a);
-    else
-      k_mean_mode<R, kMeanThreads><<<1, kMeanThreads, msm, ms>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = mark(4, ms)) != cudaSuccess) return e;
-    if (side && (e = cudaEventRecord(join, side)) != cudaSuccess) return e;
+    if (!with_inverse) {
+      const cudaStream_t ms = side ? side : s;
+      if ((e = mark(3, ms)) != cudaSuccess) return e;
+      const size_t msm = 2 * (size_t)a.Ny * sizeof(typename MeanNum<R>::T);
+      if (a.Ny <= kMeanSmallRows)
+        k_mean_mode<R, kMeanThreadsSmall><<<1, kMeanThreadsSmall, msm, ms>>>(a);
+      else
+        k_mean_mode<R, kMeanThreads><<<1, kMeanThreads, msm, ms>>>(a);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      if ((e = mark(4, ms)) != cudaSuccess) return e;
+      if (side && (e = cudaEventRecord(join, side)) != cudaSuccess) return e;
+    }
     e = (a.y_solver == 1) ? launch_modes_oddext(a, sizeof(R) == 8, s) : launch_modes(a, s);
     if (e != cudaSuccess) return e;
   }
   if ((e = mark(1, s)) != cudaSuccess) return e;
+  if (with_inverse && (e = mark(3, s)) != cudaSuccess) return e;
   if constexpr (sizeof(R) == 8) {
     e = launch_irfft64(a, false, s);
+  } else if (with_inverse) {
+    e = launch_irfft_mean(a, s);
   } else if (warp_fft) {
     e = launch_irfft_warp(a, s);
   } else {
@@ -1365,6 +1375,7 @@ cudaError_t poisson_t(const PoissonArgs& a, cudaStream_t s, cudaStream_t side, c
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) return e;
+  if (with_inverse && (e = mark(4, s)) != cudaSuccess) return e;
   if (a.ex) {
     // spectral E_x: the inverse row transform of -i k_m phi_m, formed as it
     // reads the solved spectrum

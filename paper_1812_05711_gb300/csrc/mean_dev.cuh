@@ -183,51 +183,53 @@ __device__ __forceinline__ void mean_mode_core(const PoissonArgs& a, typename Me
   }
 }
 
-template <class R, int NT>
-__device__ __forceinline__ void mean_mode_body(const PoissonArgs& a, unsigned char* smem_raw,
-                                               MeanScratch<R, NT>& ms) {
-  using N = MeanNum<R>;
-  using T = typename N::T;
+// The step's wall fluxes, added to the run's FP64 totals by threads t < NT: a
+// shuffle tree over the strips, in the warps that hold partials (the others'
+// totals would be +0, whose addition changes nothing; FP64 issue is slow on
+// this part).
+template <int NT>
+__device__ __forceinline__ void wall_flux_totals(const PoissonArgs& a, double (*fq)[NT / 32], int t) {
   constexpr int NW = NT / 32;
-  T* v = reinterpret_cast<T*>(smem_raw);  // [Ny]: s, then S, then T
-  const int Ny = a.Ny, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  if (a.flux_part) {
-    // FP64 totals of the wall fluxes: a shuffle tree over the strips, in the
-    // warps that hold partials (the others' totals would be +0, whose
-    // addition changes nothing; FP64 issue is slow on this part)
-    const int nfw = min(NW, (a.nflux + 31) / 32);
-    double qi = 0.0, qo = 0.0;
-    if (warp < nfw) {
-      for (int b = t; b < a.nflux; b += NT) {
-        qi += a.flux_part[b];
-        qo += a.flux_part[a.nflux + b];
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        qi += __shfl_down_sync(0xffffffffu, qi, o);
-        qo += __shfl_down_sync(0xffffffffu, qo, o);
-      }
+  const int lane = t & 31, warp = t >> 5;
+  const int nfw = min(NW, (a.nflux + 31) / 32);
+  double qi = 0.0, qo = 0.0;
+  if (warp < nfw) {
+    for (int b = t; b < a.nflux; b += NT) {
+      qi += __ldcg(a.flux_part + b);
+      qo += __ldcg(a.flux_part + a.nflux + b);
     }
-    auto& fq = ms.fq;
-    if (lane == 0 && warp < nfw) {
-      fq[0][warp] = qi;
-      fq[1][warp] = qo;
-    }
-    sub_sync<NT>();
-    if (t == 0) {
-      double si = 0.0, so = 0.0;
-      for (int w = 0; w < nfw; ++w) {
-        si += fq[0][w];
-        so += fq[1][w];
-      }
-      a.flux_acc[0] += si;
-      a.flux_acc[1] += so;
+    for (int o = 16; o > 0; o >>= 1) {
+      qi += __shfl_down_sync(0xffffffffu, qi, o);
+      qo += __shfl_down_sync(0xffffffffu, qo, o);
     }
   }
-  for (int j = t; j < Ny; j += NT) {
+  if (lane == 0 && warp < nfw) {
+    fq[0][warp] = qi;
+    fq[1][warp] = qo;
+  }
+  sub_sync<NT>();
+  if (t == 0) {
+    double si = 0.0, so = 0.0;
+    for (int w = 0; w < nfw; ++w) {
+      si += fq[0][w];
+      so += fq[1][w];
+    }
+    a.flux_acc[0] += si;
+    a.flux_acc[1] += so;
+  }
+}
+
+// The mean mode of a run by threads t < NT (v: 2 Ny numbers), from its row sums.
+template <class R, int NT>
+__device__ __forceinline__ void mean_mode_solve(const PoissonArgs& a, typename MeanNum<R>::T* v,
+                                                MeanScratch<R, NT>& ms, int t) {
+  using T = typename MeanNum<R>::T;
+  for (int j = t; j < a.Ny; j += NT) {
     if constexpr (sizeof(R) == 8) {
-      v[j] = static_cast<const double*>(a.spec0)[j];
+      v[j] = __ldcg(static_cast<const double*>(a.spec0) + j);
     } else {
-      v[j] = {static_cast<const float2*>(a.spec0)[j].x, static_cast<const float2*>(a.spec0)[j].y};
+      const float2 s = __ldcg(static_cast<const float2*>(a.spec0) + j);
+      v[j] = {s.x, s.y};
     }
   }
   sub_sync<NT>();
@@ -241,6 +243,13 @@ __device__ __forceinline__ void mean_mode_body(const PoissonArgs& a, unsigned ch
       Ebar[j] = ec.hi + ec.lo;
     }
   });
+}
+
+template <class R, int NT>
+__device__ __forceinline__ void mean_mode_body(const PoissonArgs& a, unsigned char* smem_raw,
+                                               MeanScratch<R, NT>& ms) {
+  if (a.flux_part) wall_flux_totals<NT>(a, ms.fq, threadIdx.x);
+  mean_mode_solve<R, NT>(a, reinterpret_cast<typename MeanNum<R>::T*>(smem_raw), ms, threadIdx.x);
 }
 
 // threads of the mean mode: 128 up to 1024 rows (shorter scans over the
