@@ -192,10 +192,10 @@ ehd_status ehd_step_profile(ehd_run* run, long n, double* ms_out);
  * each is resident and waiting when its predecessor ends: 1 the forward row
  * transform, 2 the wavenumber solve, 4 the inverse transform, 8 the step
  * kernel (march form: it stages its first rows' populations before waiting
- * for phi); the default is 15 up to 3 2^16 nodes and for FP64 compute, 4
- * between 2^19 and 2^21 nodes (1024 x 840: 39.2 us per step against 41.2 with
- * none) and 7 otherwise (2048 x 1680: 114.1 against 117.0 with none); results
- * are the same for every mask),
+ * for phi); the default is 15 up to 3 2^16 nodes and for FP64 compute, 6
+ * between 2^19 and 2^21 nodes (4 for rows of 2048) and 7 otherwise (2048 x
+ * 1680: 114.1 us per step against 117.0 with none); results are the same for
+ * every mask),
  * EHD_TUNE_FFT_CTA (FP32 rows
  * of 2048: 1, the default, one CTA of 64 threads per row; 0, one warp per
  * row), EHD_TUNE_Y_SOLVER (the y solve of the wavenumbers m >= 1: 0, the
@@ -233,8 +233,10 @@ ehd_status ehd_step_profile(ehd_run* run, long n, double* ms_out);
  * keeps one partition; the default is 4 for runs whose populations exceed
  * the L2 size and 0 otherwise; results differ in rounding order only, where
  * a row's charge is summed from slab-boundary partials).
- * Drops the run's captured graphs.  EHD_EINVAL for an unknown parameter or
- * value. */
+ * Drops the run's captured graphs; a run whose launch shape was set steps with
+ * the kernels that the parameters above describe (small runs otherwise step in
+ * other forms with the same results: their whole state on chip, or one node per
+ * thread).  EHD_EINVAL for an unknown parameter or value. */
 #define EHD_TUNE_SLAB_ROWS 1
 #define EHD_TUNE_RING_DEPTH 2
 #define EHD_TUNE_STEP_KERNEL 3

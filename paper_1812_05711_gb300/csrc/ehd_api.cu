@@ -49,6 +49,8 @@ Allocator g_alloc;
 
 constexpr double kPi = 3.141592653589793238462643383279502884;
 constexpr int kGraphSteps = 16;  // steps per captured graph (even: buffer parity)
+constexpr int kPushPdl = 15;  // its kernels are all launched programmatically
+constexpr long long kPushNodes = 1LL << 19;  // largest run that steps one node per thread
 constexpr int kResidentSteps = 4096;  // steps per launch of the on-chip form
 constexpr int kSlabShift = 4;    // default slab_shift of large runs (rows per step)
 
@@ -410,6 +412,29 @@ cudaError_t enqueue_base(ehd_run* r, int cur) {
   return e;
 }
 
+// Whether the run's steps are one node per thread (k_push): FP32-compute runs
+// of up to 2^19 nodes whose rows the warp transforms take, unless a launch shape
+// was asked for.  Against the march form, us per step: 256 x 205 10.5 / 13.7,
+// 512 x 416 16.2 / 19.6, 512 x 1000 (BF16) 27.2 / 30.0, 1024 x 300 20.3 / 23.2;
+// at 1024 x 840 both take 39, and beyond the populations leave L2, where the
+// march form's fewer bytes win.
+bool push_form(const ehd_run* r) {
+  return !r->tuned && !r->real_f64 && !r->pert && !r->ex_spectral && r->step_kernel == 0 && r->slab_shift == 0 &&
+         r->Nx >= 64 && r->Nx <= 1024 && r->Ny >= 16 && r->Ny <= 1024 && (long long)r->Nx * r->Ny <= kPushNodes;
+}
+// The Poisson solve after such a step into buffer `cur`.
+void push_poisson(const ehd_run* r, int cur, PoissonArgs* pa) {
+  pa->pdl = kPushPdl;
+  pa->g = r->g[cur];
+  pa->gplane = (long long)r->Ny * r->P;
+  pa->gstorage = r->storage;
+  pa->rch = r->rch;
+  pa->xslab = r->slab_rows;
+  pa->flux_strip = r->flux_part;
+  pa->flux_lo = static_cast<const float*>(r->rx_dn);
+  pa->flux_hi = static_cast<const float*>(r->rx_up);
+}
+
 // Charge plane of buffer `cur`, then phi (the Poisson solve).  Perturbation
 // form: the departure's charge and potential, and the base's potential.
 cudaError_t enqueue_poisson(ehd_run* r, int cur, bool with_flux) {
@@ -459,6 +484,11 @@ bool tma_form(const ehd_run* r) {
   return r->march_tma && r->tma_ok && r->cols_per_lane == 2 && !r->ex_spectral && r->step_kernel == 0;
 }
 cudaError_t launch_march_run(const ehd_run* r, const StepArgs& sa, int cur) {
+  if (push_form(r)) {
+    StepArgs pa = sa;
+    pa.pdl = kPushPdl;
+    return launch_push(pa, r->storage, r->log2Nx, r->stream);
+  }
   if (tma_form(r)) return launch_march_tma(sa, r->tma[cur], r->march_tma, r->stream);
   return launch_march(sa, r->storage, r->real_f64, r->stream);
 }
@@ -484,6 +514,7 @@ cudaError_t enqueue_step(ehd_run* r, int cur, long k) {
     sa.slab_off = march_shift(r, k);
     PoissonArgs pa = poisson_args(r, true);
     pa.xoff = sa.slab_off;
+    if (push_form(r)) push_poisson(r, 1 - cur, &pa);
     cudaError_t e = fork_base(r);
     if (e == cudaSuccess) e = launch_march_run(r, sa, cur);
     if (e == cudaSuccess) e = launch_poisson(pa, r->real_f64, r->stream, r->side, r->ev_fork, r->ev_join);
@@ -783,20 +814,24 @@ ehd_status ehd_create(int Nx, int Ny, double T, double C, double M, double Fe, d
     r->bmom = static_cast<double*>(run_alloc(r, 5 * (size_t)Ny * sizeof(double)));
   }
   r->step_kernel = (o.step_kernel >= 0) ? o.step_kernel : (r->real_f64 && !o.ex_spectral) ? 1 : 0;
-  // programmatic dependent launch (mask of EHD_TUNE_PDL), as measured per
-  // step.  FP64, and FP32 up to 3 2^16 nodes: all four kernels (15; 256 x 205:
-  // 13.7 us against 14.5 with 7 and 17.8 with none; 512 x 300: 19.0 / 19.2 /
-  // 21.5).  Up to 2^19 nodes the three Poisson kernels (7; 512 x 416: 19.6
-  // against 21.0 with 15), whose early CTAs no longer find room beside the
-  // march.  Up to 2^21 the inverse transform only, which carries the mean mode
-  // (4; 1024 x 840: 39.2 against 41.5 with 7, 41.2 with none).  Beyond, where
-  // the Poisson kernels are short against the march, all three again (7; 2048 x
-  // 1680: 114.1 against 114.7 with 6, 117.0 with none).  The perturbation form
-  // follows the same line (512 x 416: 20.3 with 7; 1024 x 840: 40.5 with 4,
-  // 44.2 with 7)
+  // programmatic dependent launch (mask of EHD_TUNE_PDL), as measured per step
+  // of the march form (runs that step one node per thread take all four).
+  // FP64, and FP32 up to 3 2^16 nodes: all four kernels (15; perturbation form
+  // 128 x 104: 15.0 us against 15.2 with 7 and 16.7 with none).  Up to 2^19
+  // nodes the three Poisson kernels (7; 512 x 416: 19.6 against 21.0 with 15).
+  // Up to 2^21 the wavenumber solve and the inverse transform, which carries
+  // the mean mode (6; 1024 x 840: 38.1 against 41.2 with 7, 39.6 with none;
+  // perturbation form 39.1 / 46.3 / 42.8), rows of 2048 the inverse only (4;
+  // 2048 x 840: 66.7 against 68.1 with 6).  Beyond, all three again (7; 2048 x
+  // 1680: 114.1 against 114.7 with 6, 117.0 with none)
   {
     const long long nodes = (long long)Nx * Ny;
-    r->pdl = (r->real_f64 || nodes <= (3LL << 16)) ? 15 : (nodes > (1LL << 19) && nodes < (1LL << 21)) ? 4 : 7;
+    if (r->real_f64 || nodes <= (3LL << 16))
+      r->pdl = 15;
+    else if (nodes > (1LL << 19) && nodes < (1LL << 21))
+      r->pdl = Nx == 2048 ? 4 : 6;
+    else
+      r->pdl = 7;
   }
   r->cols_per_lane = 2;
   r->nstrips = march_strips(Nx, r->cols_per_lane);
@@ -1188,6 +1223,7 @@ ehd_status ehd_step_profile(ehd_run* r, long n, double* ms_out) {
     PoissonArgs pa = poisson_args(r, true);
     pa.xoff = sa.slab_off;
     const int nxt = 1 - r->cur;
+    if (push_form(r)) push_poisson(r, nxt, &pa);
     if (e == cudaSuccess) e = cudaEventRecord(E[0], r->stream);
     if (e == cudaSuccess) e = fork_base(r);
     if (e == cudaSuccess)

@@ -264,8 +264,13 @@ struct PoissonArgs {
   int Nx, Ny, P, Mh, log2Nx;
   int Mp;                    // row pitch of the spectrum and pivot tables (Mh rounded up to 4)
   const void* rhoc;          // charge density, R [Ny][P]
-  const void* g;             // FP64: charge populations whose sum is the charge density (rhoc then unused), or nullptr
+  const void* g;             // charge populations that the forward transform sums (rhoc then unused), or nullptr
   long long gplane;          // elements per plane of g
+  int gstorage;              // FP32 compute after k_push: g's storage type, and its shift
+  const float* rch;
+  const float* flux_lo;      // wall rows' charge populations of k_push, [6][P] each
+  const float* flux_hi;
+  double* flux_strip;        // the strips' wall fluxes formed from them: flux_part
   const void* rhoc_dn;       // slab-boundary partials of the march form (see StepArgs), added to rhoc
   const void* rhoc_up;
   int xslab;                 // slab height of those partials; 0: rhoc is complete
@@ -499,6 +504,9 @@ int oddext_factors(int n, int* fac, int cap);
 size_t oddext_smem_bytes(int NE, bool real_f64);
 cudaError_t launch_modes_oddext(const PoissonArgs& a, bool real_f64, cudaStream_t s);
 cudaError_t oddext_set_attributes();
+// One node per thread (k_push.cu): FP32-compute runs without a base state;
+// the wall rows' charge populations go to rhoc_dn and rhoc_up
+cudaError_t launch_push(const StepArgs& a, int storage, int log2Nx, cudaStream_t s);
 // Many steps of a small FP32 run in one launch with its state on chip
 // (k_resident.cu): whether the size fits a cluster of this GPU (also sets the
 // kernel's attributes), and `steps` steps from a.fin / a.gin back into them.
@@ -513,6 +521,8 @@ bool fftw_supported(int Nx);
 cudaError_t fftw_set_tables();
 cudaError_t launch_rfft_warp(const PoissonArgs& a, cudaStream_t s);
 cudaError_t launch_irfft_warp(const PoissonArgs& a, cudaStream_t s);
+// the forward transform after k_push (rows of 64 to 512)
+cudaError_t launch_rfft_push(const PoissonArgs& a, cudaStream_t s);
 // the inverse transform and, beside it and the wavenumber solve, the mean mode
 bool irfft_mean_supported(int Nx, int Ny);
 cudaError_t launch_irfft_mean(const PoissonArgs& a, cudaStream_t s);

@@ -9,7 +9,10 @@
 // W_L^(n1 k2), the warp transposes through shared memory (padded rows), and
 // lane k2 finishes with a 32-point FFT in registers.  No CTA-wide barrier.
 // The inverse uses IFFT(Z) = conj(FFT(conj(Z))) / L.
+#include <type_traits>
+
 #include "fft_dev.cuh"
+#include "march_dev.cuh"
 #include "mean_dev.cuh"
 
 namespace ehd {
@@ -503,29 +506,11 @@ __global__ void __launch_bounds__(kCtaT, 12) k_irfft_cta(PoissonArgs a) {
 // run's rows of up to 512 reals, bound by the length of one warp's instruction
 // chain.  The same bits as rfft_warp_rows / irfft_warp_rows.
 template <int E>
-__device__ __forceinline__ void rfft_lane_row(const PoissonArgs& a, int y, const LaneFft<E>& fft,
-                                              const float2 (&wk)[E], float2* sm) {
+__device__ __forceinline__ void rfft_lane_charge(const PoissonArgs& a, int y, const float2 (&v)[E],
+                                                 const LaneFft<E>& fft, const float2 (&wk)[E], float2* sm) {
   const int lane = threadIdx.x & 31;
   constexpr int L = 32 * E, N = 2 * L;
   const float nieps = -(float)a.inv_eps;
-  const float2* rc2 = reinterpret_cast<const float2*>(static_cast<const float*>(a.rhoc) + (long long)y * a.P);
-  const float *rdn, *rup;
-  rhoc_partials<float>(a, y, rdn, rup);
-  float2 v[E];
-#pragma unroll
-  for (int n2 = 0; n2 < E; ++n2) {
-    v[n2] = rc2[lane + 32 * n2];
-    if (rdn) {
-      const float2 d = reinterpret_cast<const float2*>(rdn)[lane + 32 * n2];
-      v[n2].x += d.x;
-      v[n2].y += d.y;
-    }
-    if (rup) {
-      const float2 u = reinterpret_cast<const float2*>(rup)[lane + 32 * n2];
-      v[n2].x += u.x;
-      v[n2].y += u.y;
-    }
-  }
   const float c0 = __shfl_sync(0xffffffffu, v[0].x, 0);  // the row constant (see rfft_warp_rows)
   float re[E], im[E];
 #pragma unroll
@@ -544,6 +529,31 @@ __device__ __forceinline__ void rfft_lane_row(const PoissonArgs& a, int y, const
     spec[k] = (k == 0) ? make_float2(0.0f, 0.0f) : untangle<E>(sm, k, wk[j]);
   }
   if (lane == 0) spec[L] = make_float2(re[0] - im[0], 0.0f);  // Nyquist: Re Z0 - Im Z0
+}
+
+template <int E>
+__device__ __forceinline__ void rfft_lane_row(const PoissonArgs& a, int y, const LaneFft<E>& fft,
+                                              const float2 (&wk)[E], float2* sm) {
+  const int lane = threadIdx.x & 31;
+  const float2* rc2 = reinterpret_cast<const float2*>(static_cast<const float*>(a.rhoc) + (long long)y * a.P);
+  const float *rdn, *rup;
+  rhoc_partials<float>(a, y, rdn, rup);
+  float2 v[E];
+#pragma unroll
+  for (int n2 = 0; n2 < E; ++n2) {
+    v[n2] = rc2[lane + 32 * n2];
+    if (rdn) {
+      const float2 d = reinterpret_cast<const float2*>(rdn)[lane + 32 * n2];
+      v[n2].x += d.x;
+      v[n2].y += d.y;
+    }
+    if (rup) {
+      const float2 u = reinterpret_cast<const float2*>(rup)[lane + 32 * n2];
+      v[n2].x += u.x;
+      v[n2].y += u.y;
+    }
+  }
+  rfft_lane_charge<E>(a, y, v, fft, wk, sm);
 }
 
 template <int E, bool DX>
@@ -591,7 +601,9 @@ __global__ void __launch_bounds__(128) k_rfft_warp(PoissonArgs a) {
     if (y < a.Ny) rfft_lane_row<E>(a, y, fft, wk, smem[warp]);
   } else {
     grid_dep_wait();
-    grid_dep_launch();
+    // rows of 1024: the wavenumber solve is not released early (see
+    // k_rfft_push; 1024 x 840: 38.1 us per step against 39.2)
+    if constexpr (E > 16) grid_dep_launch();
     if (y < a.Ny) rfft_warp_rows<E, 1>(a, y, smem[warp]);
   }
 }
@@ -773,6 +785,130 @@ cudaError_t launch_rfft_warp(const PoissonArgs& a, cudaStream_t s) {
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
+}
+
+// Two adjacent populations of the storage type.
+template <class S>
+__device__ __forceinline__ float2 ld_pair(const S* p) {
+  if constexpr (sizeof(S) == 8) {
+    const double2 v = __ldg(reinterpret_cast<const double2*>(p));
+    return make_float2((float)v.x, (float)v.y);
+  } else if constexpr (sizeof(S) == 4) {
+    return __ldg(reinterpret_cast<const float2*>(p));
+  } else if constexpr (std::is_same_v<S, __half>) {
+    const float2 v = __half22float2(__ldg(reinterpret_cast<const __half2*>(p)));
+    return make_float2(v.x * kHalfUnscale, v.y * kHalfUnscale);
+  } else {
+    return __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162*>(p)));
+  }
+}
+
+// The forward transform after the one-node-per-thread step (k_push): the row's
+// charge density summed from the populations, a pair of nodes per thread (nine
+// loads in flight each; more pairs for rows of 512 and 1024) by as many warps
+// as that takes, then the transform by the first of them.  The wavenumber solve
+// is not released early: its few CTAs, resident among these, were packed onto
+// some SMs (256 x 205: 10.5 us per step or 13 to 17, by chance).
+template <int E>
+struct PushRow {
+  static constexpr int kWarps = E < 4 ? E : 4, kRows = 4 / kWarps;  // warps per row, rows per CTA
+};
+// The CTAs after the rows' form the strips' wall fluxes, a warp each, from the
+// wall rows' six charge populations that k_push leaves ([6][P] per wall;
+// injector: the three new ones and the three they came from; collector: the
+// three that leave and the three that re-enter), summed as the march form does:
+// a pair of columns of a 60-column strip per lane, then a shuffle tree.
+__device__ __forceinline__ void strip_flux(const PoissonArgs& a, int k) {
+  const int lane = threadIdx.x & 31, ns = a.nflux, P = a.P;
+  const bool hi = k >= ns;
+  const int x = 60 * (hi ? k - ns : k) + 2 * (lane - 1);
+  const float* w = hi ? a.flux_hi : a.flux_lo;
+  double q = 0.0;
+  if (lane >= 1 && lane <= 30 && x < a.Nx) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      double z[6];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) z[i] = (double)w[i * P + x + j];
+      if (hi) {
+        q += (z[0] + z[1]) + z[2];
+        q -= (z[3] + z[4]) + z[5];
+      } else {
+        q += ((z[0] - z[3]) + (z[1] - z[4])) + (z[2] - z[5]);
+      }
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) q += __shfl_down_sync(0xffffffffu, q, o);
+  if (lane == 0) a.flux_strip[k] = q;
+}
+template <class S, int E>
+__global__ void __launch_bounds__(128) k_rfft_push(PoissonArgs a) {
+  using C = PushRow<E>;
+  constexpr int L = 32 * E, T = 32 * C::kWarps;
+  __shared__ float2 smem[C::kRows][E * 34];
+  __shared__ float2 charge[C::kRows][L];
+  const int r = threadIdx.x / T, t = threadIdx.x % T, lane = threadIdx.x & 31;
+  const int y = blockIdx.x * C::kRows + r;
+  const bool live = y < a.Ny;
+  const int row_ctas = (a.Ny + C::kRows - 1) / C::kRows;
+  if ((int)blockIdx.x >= row_ctas) {
+    const int k = ((int)blockIdx.x - row_ctas) * 4 + (threadIdx.x >> 5);
+    grid_dep_wait();
+    if (k < 2 * a.nflux) strip_flux(a, k);
+    return;
+  }
+  LaneFft<E> fft;
+  float2 wk[E];
+  if (t < 32) {
+    fft.init(static_cast<const float2*>(a.tw), lane);
+    untangle_factors<E>(static_cast<const float2*>(a.tw), lane, wk);
+  }
+  const float s = live ? __ldg(a.rch + y) : 0.0f;
+  grid_dep_wait();
+  if (live) {
+    const S* __restrict__ g = static_cast<const S*>(a.g) + (long long)y * a.P;
+    const bool first = slab_first(y, a.xslab), last = slab_last(y, a.Ny, a.xslab);
+#pragma unroll
+    for (int p = t; p < L; p += T) {
+      float2 c[9];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) c[i] = ld_pair(g + i * a.gplane + 2 * p);
+      charge[r][p] = make_float2(march_charge(s, first, last, [&](int i) { return c[i].x; }),
+                                 march_charge(s, first, last, [&](int i) { return c[i].y; }));
+    }
+  }
+  __syncthreads();
+  if (!live || t >= 32) return;
+  float2 v[E];
+#pragma unroll
+  for (int n2 = 0; n2 < E; ++n2) v[n2] = charge[r][lane + 32 * n2];
+  rfft_lane_charge<E>(a, y, v, fft, wk, smem[r]);
+}
+
+namespace {
+template <class S>
+cudaError_t rfft_push_s(const PoissonArgs& a, cudaStream_t s) {
+  const dim3 b(128);
+  const unsigned n = (unsigned)a.Ny, f = (unsigned)(2 * a.nflux + 3) / 4;  // row CTAs, then the strips' flux
+  const bool pdl = (a.pdl & 1) != 0;
+  switch (a.Nx) {
+    case 64: return launch_ex(pdl, k_rfft_push<S, 1>, dim3((n + 3) / 4 + f), b, 0, s, a);
+    case 128: return launch_ex(pdl, k_rfft_push<S, 2>, dim3((n + 1) / 2 + f), b, 0, s, a);
+    case 256: return launch_ex(pdl, k_rfft_push<S, 4>, dim3(n + f), b, 0, s, a);
+    case 512: return launch_ex(pdl, k_rfft_push<S, 8>, dim3(n + f), b, 0, s, a);
+    case 1024: return launch_ex(pdl, k_rfft_push<S, 16>, dim3(n + f), b, 0, s, a);
+    default: return cudaErrorInvalidValue;
+  }
+}
+}  // namespace
+cudaError_t launch_rfft_push(const PoissonArgs& a, cudaStream_t s) {
+  switch (a.gstorage) {
+    case 0: return rfft_push_s<double>(a, s);
+    case 1: return rfft_push_s<float>(a, s);
+    case 2: return rfft_push_s<__nv_bfloat16>(a, s);
+    case 3: return rfft_push_s<__half>(a, s);
+  }
+  return cudaErrorInvalidValue;
 }
 
 // rows of 64 to 1024 with the mean mode (up to 1024 rows, 16 KB)

@@ -1321,6 +1321,8 @@ cudaError_t poisson_t(const PoissonArgs& a, cudaStream_t s, cudaStream_t side, c
   cudaError_t e;
   if constexpr (sizeof(R) == 8) {
     e = launch_rfft64(a, s);
+  } else if (a.g) {
+    e = launch_rfft_push(a, s);
   } else if (warp_fft) {
     e = launch_rfft_warp(a, s);
   } else {

@@ -324,29 +324,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(StepArgs a, PoissonArg
     // ----------------------------------------------------------- forward
     double wall = 0.0;  // this lane's share of the strip's wall flux
     if (warp < nr) {
-      // charge density, summed as the march form leaves it: a slab's last
-      // row lacks the populations pushed down into it, its first row those
-      // pushed up, until the transform adds their shares
       const float* g = q + 9 * RN + warp * Nx;
       const float s = shift[warp + 1];
-      const bool first = myrow > 0 && myrow % slab == 0, last = myrow + 1 < Ny && (myrow + 1) % slab == 0;
+      const bool first = slab_first(myrow, slab), last = slab_last(myrow, Ny, slab);
       float2 v[E];
 #pragma unroll
       for (int n2 = 0; n2 < E; ++n2) {
         float2 c[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) c[i] = *reinterpret_cast<const float2*>(g + i * RN + 2 * (lane + 32 * n2));
-        float r[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          auto z = [&](int i) { return j == 0 ? c[i].x : c[i].y; };
-          const float h = (z(0) + z(1)) + z(3), u = (z(2) + z(5)) + z(6), d = (z(4) + z(7)) + z(8);
-          const float hu = first ? h : h + u;
-          r[j] = last ? s + hu : s + (hu + d);
-          if (last) r[j] += d;
-          if (first) r[j] += u;
-        }
-        v[n2] = make_float2(r[0], r[1]);
+        v[n2] = make_float2(march_charge(s, first, last, [&](int i) { return c[i].x; }),
+                            march_charge(s, first, last, [&](int i) { return c[i].y; }));
       }
       const float c0 = __shfl_sync(0xffffffffu, v[0].x, 0);
       float re[E], im[E];

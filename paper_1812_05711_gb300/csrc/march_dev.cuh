@@ -85,4 +85,21 @@ __device__ __forceinline__ void collide_node(R (&f)[9], R (&g)[9], R Ex, R Ey, R
   trt_g2<R>(g[6], g[8], W2, drc, rc, vy - vx, vsq15, gwp, gwm);
 }
 
+// Charge density of one node from its new populations z(0) .. z(8) and the
+// shift s of its row, summed as the march form leaves it: a slab's last row
+// lacks the populations pushed down into it, its first row those pushed up,
+// until the forward transform adds their shares.
+template <class Z>
+__device__ __forceinline__ float march_charge(float s, bool first, bool last, Z&& z) {
+  const float h = (z(0) + z(1)) + z(3), u = (z(2) + z(5)) + z(6), d = (z(4) + z(7)) + z(8);
+  const float hu = first ? h : h + u;
+  float r = last ? s + hu : s + (hu + d);
+  if (last) r += d;
+  if (first) r += u;
+  return r;
+}
+// row y opens / closes a slab of S rows
+__device__ __forceinline__ bool slab_first(int y, int S) { return y > 0 && y % S == 0; }
+__device__ __forceinline__ bool slab_last(int y, int Ny, int S) { return y + 1 < Ny && (y + 1) % S == 0; }
+
 }  // namespace ehd
