@@ -140,7 +140,7 @@ struct ehd_run {
   double* phiB = nullptr;
   double* brhs = nullptr;
   double* bsum = nullptr;  // [4][Ny] rho_c, rho, j_y, j_x of the newest base state, [2][Ny] + [2][chunks] its prefix sums
-  double* bmom = nullptr;  // [5][Ny] its moments for the next base step
+  double* bmom = nullptr;  // [7][Ny] its moments for the next base step
   float* btab[2] = {nullptr, nullptr};
   cudaStream_t side2 = nullptr;  // the base chain: forked at the start of the step, joined at its end
   cudaEvent_t ev_base = nullptr, ev_start = nullptr;
@@ -358,7 +358,9 @@ BasePoissonArgs base_poisson_args(const ehd_run* r, int cur) {
   b.Nx = r->Nx;
   b.Ny = r->Ny;
   b.wall_mode = r->wall_mode;
-  b.phi0 = r->phi0;
+  b.W = (double)r->Nx * r->phi0;
+  b.closure = (r->wall_mode == 0) ? 1.0 / (2.0 * r->Ny) : 1.0 / (double)(r->Ny + 1);
+  b.inN = 1.0 / (double)r->Nx;
   b.mub = r->mub;
   b.rhs = r->brhs;
   b.sums = r->bsum;
@@ -380,15 +382,12 @@ BaseArgs base_step_args(const ehd_run* r, int cur) {
   b.gout = r->bg[1 - cur];
   b.EB = r->EBd;
   b.wp = 1.0 / r->tau_p;
-  b.wm = 1.0 / r->tau_m;
   b.gwp = 1.0 / r->taug_p;
-  b.gwm = 1.0 / r->taug_m;
+  b.k64 = collide_f64_constants(b.wp, 1.0 / r->tau_m, b.gwp, 1.0 / r->taug_m);
   b.mub = r->mub;
   b.rho0 = r->rho0;
-  b.eps = r->eps;
+  b.rhs_scale = -(double)r->Nx / r->eps;
   b.flux_acc = r->small + 8;
-  b.cp = 1.0 - 0.5 * b.wp;
-  b.cm = 1.0 - 0.5 * b.wm;
   b.mom = r->bmom;
   b.sums = r->bsum;
   b.rhs = r->brhs;
@@ -764,8 +763,8 @@ ehd_status ehd_create(int Nx, int Ny, double T, double C, double M, double Fe, d
     return fail(EHD_ECUDA, "stream/event creation failed");
   }
   {
-    cudaError_t e = poisson_set_attributes();
-    if (e == cudaSuccess) e = march_set_attributes();
+    cudaError_t e = poisson_set_attributes(r->real_f64);
+    if (e == cudaSuccess) e = march_set_attributes(r->storage, r->real_f64);
     if (e == cudaSuccess) e = oddext_set_attributes();
     if (e != cudaSuccess) {
       destroy_quiet(r);
@@ -811,7 +810,7 @@ ehd_status ehd_create(int Nx, int Ny, double T, double C, double M, double Fe, d
     r->phiB = static_cast<double*>(run_alloc(r, (size_t)Ny * sizeof(double)));
     r->brhs = static_cast<double*>(run_alloc(r, (size_t)Ny * sizeof(double)));
     r->bsum = static_cast<double*>(run_alloc(r, (6 * (size_t)Ny + 2 * (size_t)base_chunks(Ny)) * sizeof(double)));
-    r->bmom = static_cast<double*>(run_alloc(r, 5 * (size_t)Ny * sizeof(double)));
+    r->bmom = static_cast<double*>(run_alloc(r, 7 * (size_t)Ny * sizeof(double)));
   }
   r->step_kernel = (o.step_kernel >= 0) ? o.step_kernel : (r->real_f64 && !o.ex_spectral) ? 1 : 0;
   // programmatic dependent launch (mask of EHD_TUNE_PDL), as measured per step
@@ -1608,8 +1607,8 @@ ehd_status ehd_batch_create(int max_runs, size_t hbm_budget, int max_nx, int max
     return fail(EHD_ECUDA, "stream/event creation failed");
   }
   {
-    cudaError_t e = poisson_set_attributes();
-    if (e == cudaSuccess) e = march_set_attributes();
+    cudaError_t e = poisson_set_attributes(false);
+    if (e == cudaSuccess) e = march_set_attributes(-1, false);
     if (e != cudaSuccess) {
       batch_free(b);
       return fail(EHD_ECUDA, "kernel attributes: %s", cudaGetErrorString(e));

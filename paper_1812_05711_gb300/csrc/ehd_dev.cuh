@@ -380,9 +380,10 @@ struct BaseArgs {
   double* fout;        // [9][Ny] at t + 1
   double* gout;
   const double* EB;    // [Ny] base E_y at time t
-  const double* mom;   // [5][Ny] rho, rho_c, u_x, u_y, u_y + mu_b E_y at time t
-  double wp, wm, gwp, gwm, mub, rho0, eps;
-  double cp, cm;       // force factors 1 - wp / 2, 1 - wm / 2
+  const double* mom;   // [7][Ny] rho_c, rho, u_x, u_y, u_y + mu_b E_y, j_x, j_y at time t
+  double wp, gwp, mub, rho0;
+  double rhs_scale;    // -Nx / eps
+  CollideF64 k64;
   double* flux_acc;    // [2] FP64 totals of the base's injected / collected charge
   double* sums;        // [4][Ny] rho_c, rho, j_y, j_x of the state at t + 1 (out)
   double* rhs;         // [Ny] its mean-mode right-hand side -Nx rho_c / eps (out)
@@ -391,7 +392,8 @@ struct BaseArgs {
 };
 struct BasePoissonArgs {
   int Nx, Ny, wall_mode;
-  double phi0, mub;
+  double W, closure, inN;  // Nx phi0, 1 / (2 Ny) (walls halfway) or 1 / (Ny + 1), 1 / Nx
+  double mub;
   const double* rhs;   // [Ny] mean-mode right-hand side of the state
   const double* sums;  // [4][Ny] its rho_c, rho, j_y, j_x
   const double* loc;   // [2][Ny] and the chunk sums of the right-hand side
@@ -399,7 +401,7 @@ struct BasePoissonArgs {
   double* phiB;        // [Ny] base potential (out)
   double* EB;          // [Ny] base E_y (out)
   float* table;        // [Ny][4] march table (out)
-  double* mom;         // [5][Ny] moments for the state's base step (out)
+  double* mom;         // [7][Ny] moments for the state's base step (out)
 };
 // rows per chunk of the base kernels: chunks of a run's base state
 int base_chunks(int Ny);
@@ -488,7 +490,8 @@ int step_flux_blocks(int Nx, bool real_f64);
 cudaError_t launch_march(const StepArgs& a, int storage, bool real_f64, cudaStream_t s);
 int march_strips(int Nx, int cols_per_lane);
 int march_warps_per_sm(int storage, bool real_f64, int cols_per_lane, int ring_depth);
-cudaError_t march_set_attributes();
+// kernel attributes and tables for runs of this kind (storage < 0: the batch's)
+cudaError_t march_set_attributes(int storage, bool real_f64);
 // Poisson solve from the charge plane: forward row FFTs and the wavenumber
 // systems on s; the FP64 mean mode (and the wall-flux totals) on `side`
 // between the fork and join events when side != nullptr.
@@ -515,7 +518,7 @@ cudaError_t launch_resident(const StepArgs& a, const PoissonArgs& pa, int storag
 // rho_c = sum_i g_i (+ the row shift) into the charge plane (FP32 compute).
 cudaError_t launch_rhoc(const void* g, long long plane, int storage, int Nx, int Ny, int P,
                         const float* rch, void* rhoc, cudaStream_t s);
-cudaError_t poisson_set_attributes();
+cudaError_t poisson_set_attributes(bool real_f64);
 // warp-per-row real FFTs (FP32 path, Nx = 64 ... 2048)
 bool fftw_supported(int Nx);
 cudaError_t fftw_set_tables();

@@ -835,22 +835,6 @@ __device__ __forceinline__ double bw(int i) { return i == 0 ? kW0 : (i < 5 ? kW1
 __device__ __forceinline__ int bcx(int i) { return (i == 1 || i == 5 || i == 8) ? 1 : ((i == 3 || i == 6 || i == 7) ? -1 : 0); }
 __device__ __forceinline__ int bcy(int i) { return (i == 2 || i == 5 || i == 6) ? 1 : ((i == 4 || i == 7 || i == 8) ? -1 : 0); }
 __device__ __forceinline__ int bopp(int i) { return i == 0 ? 0 : (i < 5 ? ((i + 1) & 3) + 1 : ((i - 3) & 3) + 5); }
-// c_q . v with the lattice direction known at compile time
-template <int Q>
-__device__ __forceinline__ double bcdot(double vx, double vy) {
-  constexpr int cx = (Q == 1 || Q == 5 || Q == 8) ? 1 : ((Q == 3 || Q == 6 || Q == 7) ? -1 : 0);
-  constexpr int cy = (Q == 2 || Q == 5 || Q == 6) ? 1 : ((Q == 4 || Q == 7 || Q == 8) ? -1 : 0);
-  if constexpr (cx == 0 && cy == 0) return 0.0;
-  else if constexpr (cx == 0) return cy > 0 ? vy : -vy;
-  else if constexpr (cy == 0) return cx > 0 ? vx : -vx;
-  else return (cx > 0 ? vx : -vx) + (cy > 0 ? vy : -vy);
-}
-// equilibrium (Eq. 12 / 14) with |v|^2 passed in
-template <int Q>
-__device__ __forceinline__ double beq(double dens, double vx, double vy, double v2) {
-  const double cu = bcdot<Q>(vx, vy);
-  return bw(Q) * dens * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * v2);
-}
 constexpr int kBaseRows = 30;
 // the groups' populations: {0, 1, 3}, {2, 4}, {5, 7}, {6, 8}
 __device__ __forceinline__ int bgroup_pop(int grp, int k) {
@@ -865,47 +849,60 @@ struct BaseSmem {
   double qin[3];                // injected-charge terms of the populations 2, 5, 6
 };
 
-// The TRT collision of the population pair (I, O = opposite of I; I == O
-// for the rest population).  The odd parts of the pair are equal and
-// opposite, so one set of half sums serves both.  The force has no x part
-// (E_x = 0 in an x-uniform state): F_i = w_i (3 (c_iy - u_y) + 9 (c_i.u) c_iy) F_y.
+// A row's terms of collide_f64 (see there), with F_x = 0 (E_x = 0 in an
+// x-uniform state): what the four warps of a row share, about 20 FP64
+// instructions, before each collides its own pairs with about 25.
 struct BaseRow {
-  double rho, rc, ux, uy, vy, Fy, u2, v2;
+  double ux, uy, vy;
+  double C, Q, Gx, Gy, Jx, Jy;       // fluid
+  double gC, gQ, gGx, gGy, gJx, gJy;  // charge
 };
-template <int I, int O>
-__device__ __forceinline__ void base_collide_pair(const BaseArgs& a, const BaseRow& b, int y, BaseSmem& sm,
-                                                  int lane) {
+__device__ __forceinline__ BaseRow base_row(const BaseArgs& a, int y) {
+  constexpr double third = -1.0 / 3.0;
   const int Ny = a.Ny;
+  const CollideF64& k = a.k64;
+  BaseRow b;
+  const double rc = a.mom[y], rho = a.mom[Ny + y];
+  b.ux = a.mom[2 * Ny + y];
+  b.uy = a.mom[3 * Ny + y];
+  b.vy = a.mom[4 * Ny + y];
+  const double jx = a.mom[5 * Ny + y], jy = a.mom[6 * Ny + y];
+  const double Fy = rc * a.EB[y];
+  b.Gx = k.gj * jx;
+  b.Gy = fma(k.gj, jy, k.gF * Fy);
+  b.Q = fma(b.uy, b.Gy, b.ux * b.Gx);
+  b.C = fma(third, b.Q, k.rw * rho);
+  b.Jx = k.jj * jx;
+  b.Jy = fma(k.jj, jy, k.jF * Fy);
+  const double h = k.gg * rc, m = k.gjm * rc;
+  b.gGx = h * b.ux;
+  b.gGy = h * b.vy;
+  b.gQ = fma(b.vy, b.gGy, b.ux * b.gGx);
+  b.gC = fma(third, b.gQ, k.grw * rc);
+  b.gJx = m * b.ux;
+  b.gJy = m * b.vy;
+  return b;
+}
+// The pair (I, O) of opposite populations with even part E and odd part J.
+template <int I, int O>
+__device__ __forceinline__ void base_pair(const BaseArgs& a, int y, BaseSmem& sm, int lane, double E, double J,
+                                          double gE, double gJ) {
+  const int Ny = a.Ny;
+  const CollideF64& k = a.k64;
   const double fI = a.fin[I * Ny + y], fO = a.fin[O * Ny + y];
   const double gI = a.gin[I * Ny + y], gO = a.gin[O * Ny + y];
-  const double feqI = beq<I>(b.rho, b.ux, b.uy, b.u2), feqO = beq<O>(b.rho, b.ux, b.uy, b.u2);
-  const double geqI = beq<I>(b.rc, b.ux, b.vy, b.v2), geqO = beq<O>(b.rc, b.ux, b.vy, b.v2);
-  constexpr int cyI = (I == 2 || I == 5 || I == 6) ? 1 : ((I == 4 || I == 7 || I == 8) ? -1 : 0);
-  const double cuI = bcdot<I>(b.ux, b.uy);
-  // F_O = w (3 (-c_y - u_y) + 9 (-c.u)(-c_y)) F_y
-  double FiI, FiO;
-  if constexpr (cyI == 0) {
-    FiI = bw(I) * ((0.0 - b.uy) * 3.0 * b.Fy);
-    FiO = bw(O) * ((0.0 - b.uy) * 3.0 * b.Fy);
-  } else {
-    const double c = (double)cyI;
-    FiI = bw(I) * (((c - b.uy) * 3.0 + cuI * c * 9.0) * b.Fy);
-    FiO = bw(O) * (((-c - b.uy) * 3.0 + cuI * c * 9.0) * b.Fy);
-  }
-  const double fpl = 0.5 * (fI + fO), fmi = 0.5 * (fI - fO);
-  const double epl = 0.5 * (feqI + feqO), emi = 0.5 * (feqI - feqO);
-  const double Fpl = 0.5 * (FiI + FiO), Fmi = 0.5 * (FiI - FiO);
-  const double ev = a.wp * (fpl - epl), od = a.wm * (fmi - emi);
-  const double Fe = a.cp * Fpl, Fo = a.cm * Fmi;
-  sm.fp[I][lane] = fI - ev - od + Fe + Fo;
-  const double gpl = 0.5 * (gI + gO), gmi = 0.5 * (gI - gO);
-  const double hpl = 0.5 * (geqI + geqO), hmi = 0.5 * (geqI - geqO);
-  const double gev = a.gwp * (gpl - hpl), god = a.gwm * (gmi - hmi);
-  sm.gp[I][lane] = gI - gev - god;
-  if constexpr (I != O) {
-    sm.fp[O][lane] = fO - ev + od + Fe - Fo;
-    sm.gp[O][lane] = gO - gev + god;
-  }
+  const double P = fma(k.hp, fI + fO, E), D = fma(k.hm, fI - fO, J);
+  const double gP = fma(k.ghp, gI + gO, gE), gD = fma(k.ghm, gI - gO, gJ);
+  sm.fp[I][lane] = P + D;
+  sm.fp[O][lane] = P - D;
+  sm.gp[I][lane] = gP + gD;
+  sm.gp[O][lane] = gP - gD;
+}
+// The rest populations: f + (4 C - omega+ f), the bracket small.
+__device__ __forceinline__ void base_rest(const BaseArgs& a, const BaseRow& b, int y, BaseSmem& sm, int lane) {
+  const double f = a.fin[y], g = a.gin[y];
+  sm.fp[0][lane] = f + fma(-a.wp, f, 4.0 * b.C);
+  sm.gp[0][lane] = g + fma(-a.gwp, g, 4.0 * b.gC);
 }
 
 // The mean mode of the base's Poisson equation is a double prefix sum of the
@@ -945,23 +942,27 @@ __device__ __noinline__ void base_step_cta(const BaseArgs& a, int y0, BaseSmem& 
   const int y = y0 - 1 + lane;
   const int npop = grp == 0 ? 3 : 2;
   if (y >= 0 && y < Ny) {
-    BaseRow b;
-    b.rho = a.mom[y];
-    b.rc = a.mom[Ny + y];
-    b.ux = a.mom[2 * Ny + y];
-    b.uy = a.mom[3 * Ny + y];
-    b.vy = a.mom[4 * Ny + y];
-    b.Fy = b.rc * a.EB[y];
-    b.u2 = b.ux * b.ux + b.uy * b.uy;
-    b.v2 = b.ux * b.ux + b.vy * b.vy;
+    const BaseRow b = base_row(a, y);
     switch (grp) {
       case 0:
-        base_collide_pair<0, 0>(a, b, y, sm, lane);
-        base_collide_pair<1, 3>(a, b, y, sm, lane);
+        base_rest(a, b, y, sm, lane);
+        base_pair<1, 3>(a, y, sm, lane, fma(b.ux, b.Gx, b.C), b.Jx, fma(b.ux, b.gGx, b.gC), b.gJx);
         break;
-      case 1: base_collide_pair<2, 4>(a, b, y, sm, lane); break;
-      case 2: base_collide_pair<5, 7>(a, b, y, sm, lane); break;
-      default: base_collide_pair<6, 8>(a, b, y, sm, lane); break;
+      case 1:
+        base_pair<2, 4>(a, y, sm, lane, fma(b.uy, b.Gy, b.C), b.Jy, fma(b.vy, b.gGy, b.gC), b.gJy);
+        break;
+      default: {
+        // diagonals: a quarter of C + Q +- X and of J_y +- J_x (+ for 5, 7)
+        const double q = grp == 2 ? 0.25 : -0.25;
+        const double X = fma(b.ux, b.Gy, b.uy * b.Gx), gX = b.ux * b.gGy;
+        const double E = fma(q, X, 0.25 * (b.C + b.Q)), J = fma(q, b.Jx, 0.25 * b.Jy);
+        const double gE = fma(2.0 * q, gX, 0.25 * (b.gC + b.gQ)), gJ = fma(q, b.gJx, 0.25 * b.gJy);
+        if (grp == 2)
+          base_pair<5, 7>(a, y, sm, lane, E, J, gE, gJ);
+        else
+          base_pair<6, 8>(a, y, sm, lane, E, J, gE, gJ);
+        break;
+      }
     }
   }
   __syncthreads();
@@ -1011,7 +1012,7 @@ __device__ __noinline__ void base_step_cta(const BaseArgs& a, int y0, BaseSmem& 
       double rc = 0;
       for (int i = 0; i < 9; ++i) rc += sm.ng[i][lane];
       a.sums[y] = rc;
-      s = -(double)a.Nx * rc / a.eps;
+      s = a.rhs_scale * rc;
       a.rhs[y] = s;
     }
     base_chunk_scan(s, out, lane, y0 / kBaseRows, y, a.loc, a.chunk, Ny);
@@ -1022,13 +1023,11 @@ __device__ __noinline__ void base_step_cta(const BaseArgs& a, int y0, BaseSmem& 
       for (int i = 0; i < 9; ++i) rho += sm.nf[i][lane];
       a.sums[Ny + y] = rho;
     } else if (grp == 1) {
-      double jy = 0;
-      for (int i = 0; i < 9; ++i) jy += bcy(i) * sm.nf[i][lane];
-      a.sums[2 * Ny + y] = jy;
+      a.sums[2 * Ny + y] = (sm.nf[2][lane] - sm.nf[4][lane]) + (sm.nf[5][lane] - sm.nf[7][lane]) +
+                           (sm.nf[6][lane] - sm.nf[8][lane]);
     } else if (grp == 3) {
-      double jx = 0;
-      for (int i = 0; i < 9; ++i) jx += bcx(i) * sm.nf[i][lane];
-      a.sums[3 * Ny + y] = jx;
+      a.sums[3 * Ny + y] = (sm.nf[1][lane] - sm.nf[3][lane]) + (sm.nf[5][lane] - sm.nf[7][lane]) -
+                           (sm.nf[6][lane] - sm.nf[8][lane]);
     }
     if (grp == 3 && y == 0) {
       // injected charge: the down-movers 4, 7, 8 reflected into 2, 5, 6
@@ -1068,7 +1067,7 @@ __global__ void __launch_bounds__(32) k_base_sums(BaseArgs a) {
     a.sums[Ny + y] = rho;
     a.sums[2 * Ny + y] = jy;
     a.sums[3 * Ny + y] = jx;
-    s = -(double)a.Nx * rc / a.eps;
+    s = a.rhs_scale * rc;
     a.rhs[y] = s;
   }
   base_chunk_scan(s, valid, lane, c, y, a.loc, a.chunk, Ny);
@@ -1140,14 +1139,14 @@ __device__ __noinline__ void base_potential_warp(const BasePoissonArgs& b, int c
   const double S_last = S0L + b.loc[Ny - 1];
   const double T_last = (T0L + (double)(Ny - 1 - jL) * S0L) + b.loc[Ny + Ny - 1];
   const double T_all = T_last + S_last;
-  const double W = (double)b.Nx * b.phi0;
+  const double W = b.W;
   double Dm, Pm;
   if (b.wall_mode == 0) {
     const double num = (W + W) + (T_all + T_last);
-    Dm = -num * (1.0 / (2.0 * Ny));
-    Pm = W + -(Dm * 0.5);
+    Dm = -num * b.closure;
+    Pm = fma(-0.5, Dm, W);
   } else {
-    Dm = -(W + T_all) * (1.0 / (double)(Ny + 1));
+    Dm = -(W + T_all) * b.closure;
     Pm = W;
   }
   const int j0 = c * kBaseRows, j = j0 + lane;
@@ -1159,18 +1158,20 @@ __device__ __noinline__ void base_potential_warp(const BasePoissonArgs& b, int c
     const double Tj = (T0c + (double)(j - j0) * S0c) + b.loc[Ny + j];
     const double phi = (Pm + (double)(j + 1) * Dm) + Tj;
     const double ey = -0.5 * ((Dm + Dm) + (Sj + Sjm1));
-    const double inN = 1.0 / (double)b.Nx;
-    b.phiB[j] = phi * inN;
-    const double Ey = ey * inN;
+    b.phiB[j] = phi * b.inN;
+    const double Ey = ey * b.inN;
     b.EB[j] = Ey;
     // moments of the state for its next base step (Eq. 7 with F = rho_c E_y e_y)
     const double rc = b.sums[j], rho = b.sums[Ny + j], jy = b.sums[2 * Ny + j], jx = b.sums[3 * Ny + j];
-    const double ux = jx / rho, uy = (jy + 0.5 * (rc * Ey)) / rho;
-    b.mom[j] = rho;
-    b.mom[Ny + j] = rc;
+    const double irho = recip_f64(rho);
+    const double ux = jx * irho, uy = fma(0.5, rc * Ey, jy) * irho;
+    b.mom[j] = rc;
+    b.mom[Ny + j] = rho;
     b.mom[2 * Ny + j] = ux;
     b.mom[3 * Ny + j] = uy;
-    b.mom[4 * Ny + j] = uy + b.mub * Ey;
+    b.mom[4 * Ny + j] = fma(b.mub, Ey, uy);
+    b.mom[5 * Ny + j] = jx;
+    b.mom[6 * Ny + j] = jy;
     b.table[4 * j + 0] = (float)rc;
     b.table[4 * j + 1] = (float)uy;
     b.table[4 * j + 2] = (float)Ey;
@@ -1464,13 +1465,12 @@ cudaError_t launch_batch_mean(const BatchTables& t, int step, int grid, cudaStre
   return cudaGetLastError();
 }
 
-cudaError_t poisson_set_attributes() {
+cudaError_t poisson_set_attributes(bool real_f64) {
+  if (real_f64) return set_attrs_t<double>();
   cudaError_t e = fftw_set_tables();
   if (e != cudaSuccess) return e;
   if ((e = allow_max_dynamic_smem(k_batch_modes)) != cudaSuccess) return e;
   if ((e = allow_max_dynamic_smem(k_batch_mean)) != cudaSuccess) return e;
-  e = set_attrs_t<double>();
-  if (e != cudaSuccess) return e;
   return set_attrs_t<float>();
 }
 
