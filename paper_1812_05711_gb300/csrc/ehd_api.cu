@@ -401,7 +401,9 @@ BaseArgs base_step_args(const ehd_run* r, int cur) {
 // with it (fork_base, before the march) and runs beside all of it: the chain
 // of FP64 instructions is as long as a small run's whole step (128 x 104: 15.1
 // us per step against 25.8 when forked after the forward row transform,
-// 512 x 416: 20.1 / 29.0, 2048 x 1680: 115.5 / 120.5).
+// 512 x 416: 20.1 / 29.0, 2048 x 1680: 115.5 / 120.5).  With its instructions
+// halved (k_base_step) these take 12.7, 19.9 and 114.4; at 1024 x 840 (40.6)
+// the shorter chain gained nothing: it was already hidden.
 cudaError_t fork_base(ehd_run* r) { return r->pert ? cudaEventRecord(r->ev_start, r->stream) : cudaSuccess; }
 cudaError_t enqueue_base(ehd_run* r, int cur) {
   cudaError_t e = cudaStreamWaitEvent(r->side2, r->ev_start, 0);
@@ -763,8 +765,8 @@ ehd_status ehd_create(int Nx, int Ny, double T, double C, double M, double Fe, d
     return fail(EHD_ECUDA, "stream/event creation failed");
   }
   {
-    cudaError_t e = poisson_set_attributes(r->real_f64);
-    if (e == cudaSuccess) e = march_set_attributes(r->storage, r->real_f64);
+    cudaError_t e = poisson_set_attributes();
+    if (e == cudaSuccess) e = march_set_attributes();
     if (e == cudaSuccess) e = oddext_set_attributes();
     if (e != cudaSuccess) {
       destroy_quiet(r);
@@ -1607,8 +1609,8 @@ ehd_status ehd_batch_create(int max_runs, size_t hbm_budget, int max_nx, int max
     return fail(EHD_ECUDA, "stream/event creation failed");
   }
   {
-    cudaError_t e = poisson_set_attributes(false);
-    if (e == cudaSuccess) e = march_set_attributes(-1, false);
+    cudaError_t e = poisson_set_attributes();
+    if (e == cudaSuccess) e = march_set_attributes();
     if (e != cudaSuccess) {
       batch_free(b);
       return fail(EHD_ECUDA, "kernel attributes: %s", cudaGetErrorString(e));

@@ -491,7 +491,7 @@ cudaError_t launch_march(const StepArgs& a, int storage, bool real_f64, cudaStre
 int march_strips(int Nx, int cols_per_lane);
 int march_warps_per_sm(int storage, bool real_f64, int cols_per_lane, int ring_depth);
 // kernel attributes and tables for runs of this kind (storage < 0: the batch's)
-cudaError_t march_set_attributes(int storage, bool real_f64);
+cudaError_t march_set_attributes();
 // Poisson solve from the charge plane: forward row FFTs and the wavenumber
 // systems on s; the FP64 mean mode (and the wall-flux totals) on `side`
 // between the fork and join events when side != nullptr.
@@ -518,7 +518,7 @@ cudaError_t launch_resident(const StepArgs& a, const PoissonArgs& pa, int storag
 // rho_c = sum_i g_i (+ the row shift) into the charge plane (FP32 compute).
 cudaError_t launch_rhoc(const void* g, long long plane, int storage, int Nx, int Ny, int P,
                         const float* rch, void* rhoc, cudaStream_t s);
-cudaError_t poisson_set_attributes(bool real_f64);
+cudaError_t poisson_set_attributes();
 // warp-per-row real FFTs (FP32 path, Nx = 64 ... 2048)
 bool fftw_supported(int Nx);
 cudaError_t fftw_set_tables();

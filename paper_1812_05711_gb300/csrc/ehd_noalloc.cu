@@ -297,10 +297,10 @@ __global__ void __launch_bounds__(256) k_na_inv(int Nx, int Ny, float* __restric
 // The whole solve by one cluster of 16 CTAs, for grids whose spectrum fits
 // their shared memory (64 to 512 columns, up to 2^18 nodes).  A small solve is
 // bound by its launches and by the chain of each kernel, not by the work: the
-// three kernels above take 26.6 us a call at 256 x 208 (radix-2 rows with a
+// three kernels above take 24.6 us a call at 256 x 208 (radix-2 rows with a
 // barrier a stage, an FP64 elimination of the mean mode), of which the data
-// would take 0.1; this one takes 12.3 (64 x 56: 17.7 -> 7.4; 512 x 416: 32.8 ->
-// 26.6, the last size where 16 SMs are enough).  Here a warp transforms a row (LaneFft), the wavenumbers'
+// would take 0.1; this one takes 12.3 (64 x 56: 16.4 -> 7.7; 512 x 416: 32.8 ->
+// 26.1, the last size where 16 SMs are enough).  Here a warp transforms a row (LaneFft), the wavenumbers'
 // columns are written into the CTA that solves them and back into the rows'
 // owners, and the mean mode is the FP64 double prefix sum of the run's solver.
 namespace na {

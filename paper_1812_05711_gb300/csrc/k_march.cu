@@ -1617,6 +1617,8 @@ cudaError_t attrs_t() {
     if ((e = allow_smem(k_march2<S, R, 3, false, true>)) != cudaSuccess) return e;
     if ((e = allow_smem(k_march2<S, R, 4, false, true>)) != cudaSuccess) return e;
   }
+  if ((e = allow_smem(k_batch_march<false>)) != cudaSuccess) return e;
+  if ((e = allow_smem(k_batch_march<true>)) != cudaSuccess) return e;
   if ((e = allow_smem(k_march2<S, R, 2>)) != cudaSuccess) return e;
   if ((e = allow_smem(k_march2<S, R, 2, true>)) != cudaSuccess) return e;
   if ((e = allow_smem(k_march2<S, R, 3>)) != cudaSuccess) return e;
@@ -1657,21 +1659,16 @@ int march_warps_per_sm(int storage, bool real_f64, int cols_per_lane, int ring_d
 
 int march_strips(int Nx, int cols_per_lane) { return cols_per_lane == 2 ? (Nx + 59) / 60 : (Nx + 29) / 30; }
 
-cudaError_t march_set_attributes(int storage, bool real_f64) {
+cudaError_t march_set_attributes() {
   cudaError_t e;
-  if (real_f64) return attrs_t<double, double>();
-  switch (storage) {
-    case 0: return attrs_t<double, float>();
-    case 2: return attrs_t<__nv_bfloat16, float>();
-    case 3: return attrs_t<__half, float>();
-    case 1:
-      if ((e = allow_smem(k_march_tma<2, true>)) != cudaSuccess) return e;
-      if ((e = allow_smem(k_march_tma<2, false>)) != cudaSuccess) return e;
-      if ((e = allow_smem(k_march_tma<3, false>)) != cudaSuccess) return e;
-      return attrs_t<float, float>();
-  }
-  if ((e = allow_smem(k_batch_march<false>)) != cudaSuccess) return e;
-  return allow_smem(k_batch_march<true>);
+  if ((e = allow_smem(k_march_tma<2, true>)) != cudaSuccess) return e;
+  if ((e = allow_smem(k_march_tma<2, false>)) != cudaSuccess) return e;
+  if ((e = allow_smem(k_march_tma<3, false>)) != cudaSuccess) return e;
+  if ((e = attrs_t<double, double>()) != cudaSuccess) return e;
+  if ((e = attrs_t<double, float>()) != cudaSuccess) return e;
+  if ((e = attrs_t<float, float>()) != cudaSuccess) return e;
+  if ((e = attrs_t<__nv_bfloat16, float>()) != cudaSuccess) return e;
+  return attrs_t<__half, float>();
 }
 
 cudaError_t launch_march(const StepArgs& a, int storage, bool real_f64, cudaStream_t s) {

@@ -1465,12 +1465,13 @@ cudaError_t launch_batch_mean(const BatchTables& t, int step, int grid, cudaStre
   return cudaGetLastError();
 }
 
-cudaError_t poisson_set_attributes(bool real_f64) {
-  if (real_f64) return set_attrs_t<double>();
+cudaError_t poisson_set_attributes() {
   cudaError_t e = fftw_set_tables();
   if (e != cudaSuccess) return e;
   if ((e = allow_max_dynamic_smem(k_batch_modes)) != cudaSuccess) return e;
   if ((e = allow_max_dynamic_smem(k_batch_mean)) != cudaSuccess) return e;
+  e = set_attrs_t<double>();
+  if (e != cudaSuccess) return e;
   return set_attrs_t<float>();
 }
 
