@@ -402,8 +402,9 @@ BaseArgs base_step_args(const ehd_run* r, int cur) {
 // of FP64 instructions is as long as a small run's whole step (128 x 104: 15.1
 // us per step against 25.8 when forked after the forward row transform,
 // 512 x 416: 20.1 / 29.0, 2048 x 1680: 115.5 / 120.5).  With its instructions
-// halved (k_base_step) these take 12.7, 19.9 and 114.4; at 1024 x 840 (40.6)
-// the shorter chain gained nothing: it was already hidden.
+// halved (k_base_step), on one machine: 128 x 104 15.15 -> 12.5, 512 x 416 20.5
+// -> 20.1, 1024 x 840 40.7 -> 40.5, 2048 x 1680 115.5 -> 114.0: from 512
+// columns the chain was nearly hidden already.
 cudaError_t fork_base(ehd_run* r) { return r->pert ? cudaEventRecord(r->ev_start, r->stream) : cudaSuccess; }
 cudaError_t enqueue_base(ehd_run* r, int cur) {
   cudaError_t e = cudaStreamWaitEvent(r->side2, r->ev_start, 0);
@@ -818,11 +819,11 @@ ehd_status ehd_create(int Nx, int Ny, double T, double C, double M, double Fe, d
   // programmatic dependent launch (mask of EHD_TUNE_PDL), as measured per step
   // of the march form (runs that step one node per thread take all four).
   // FP64, and FP32 up to 3 2^16 nodes: all four kernels (15; perturbation form
-  // 128 x 104: 15.0 us against 15.2 with 7 and 16.7 with none).  Up to 2^19
+  // 128 x 104: 12.8 us against 13.1 with 7).  Up to 2^19
   // nodes the three Poisson kernels (7; 512 x 416: 19.6 against 21.0 with 15).
   // Up to 2^21 the wavenumber solve and the inverse transform, which carries
   // the mean mode (6; 1024 x 840: 38.1 against 41.2 with 7, 39.6 with none;
-  // perturbation form 39.1 / 46.3 / 42.8), rows of 2048 the inverse only (4;
+  // perturbation form 40.6 / 42.6 / 43.2), rows of 2048 the inverse only (4;
   // 2048 x 840: 66.7 against 68.1 with 6).  Beyond, all three again (7; 2048 x
   // 1680: 114.1 against 114.7 with 6, 117.0 with none)
   {
