@@ -114,6 +114,7 @@ struct ehd_run {
   ModesTma mtma = {};
   bool mtma_ok = false;
   int resident = -1;   // small FP32 runs step with the whole state on chip (k_resident.cu): -1 not looked at yet
+  bool after_on_chip = false;  // the populations' last writer was k_resident: see step_pdl
   bool tuned = false;  // a launch shape was asked for (ehd_tune): the kernel-per-phase step
   int pdl = 0;         // programmatic dependent launch between the Poisson kernels (off: see ehd_tune)
   int fft_cta = 1;     // rows of 2048: CTA-per-row transforms
@@ -253,6 +254,15 @@ ehd_status upload(ehd_run* r, void* dst, const void* src, size_t bytes) {
   return EHD_OK;
 }
 
+bool push_form(const ehd_run* r);
+// Launch mask of the run's step kernel.  Bit 8, its programmatic launch, is
+// safe only where a Poisson solve lies between the kernel and the populations'
+// last writer: the step kernels read the populations before they wait, because
+// the solve, which has waited for that writer, is what they are released by.
+// k_resident writes them itself as its last act, so the step after it is
+// launched in plain stream order.
+int step_pdl(const ehd_run* r) { return (push_form(r) ? kPushPdl : r->pdl) & (r->after_on_chip ? ~8 : ~0); }
+
 StepArgs step_args(const ehd_run* r, int cur) {
   StepArgs a{};
   a.Nx = r->Nx;
@@ -286,7 +296,7 @@ StepArgs step_args(const ehd_run* r, int cur) {
   a.nstrips = r->nstrips;
   a.ring_depth = r->ring_depth;
   a.cols_per_lane = r->cols_per_lane;
-  a.pdl = r->pdl;
+  a.pdl = step_pdl(r);
   a.base_tab = r->pert ? r->btab[cur] : nullptr;
   return a;
 }
@@ -486,11 +496,7 @@ bool tma_form(const ehd_run* r) {
   return r->march_tma && r->tma_ok && r->cols_per_lane == 2 && !r->ex_spectral && r->step_kernel == 0;
 }
 cudaError_t launch_march_run(const ehd_run* r, const StepArgs& sa, int cur) {
-  if (push_form(r)) {
-    StepArgs pa = sa;
-    pa.pdl = kPushPdl;
-    return launch_push(pa, r->storage, r->log2Nx, r->stream);
-  }
+  if (push_form(r)) return launch_push(sa, r->storage, r->log2Nx, r->stream);
   if (tma_form(r)) return launch_march_tma(sa, r->tma[cur], r->march_tma, r->stream);
   return launch_march(sa, r->storage, r->real_f64, r->stream);
 }
@@ -553,10 +559,13 @@ ehd_status build_graph(ehd_run* r, int cur) {
   EHD_CK(cudaStreamBeginCapture(r->stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
   int c = cur;
+  const bool on_chip_before = r->after_on_chip;
+  r->after_on_chip = false;  // a graph starts when all before it has ended
   for (int k = 0; k < kGraphSteps && e == cudaSuccess; ++k) {
     e = enqueue_step(r, c, k);
     c = 1 - c;
   }
+  r->after_on_chip = on_chip_before;
   cudaError_t e2 = cudaStreamEndCapture(r->stream, &g);
   if (e != cudaSuccess || e2 != cudaSuccess) {
     if (g) cudaGraphDestroy(g);
@@ -1183,6 +1192,7 @@ ehd_status ehd_step(ehd_run* r, long n) {
     while (n > 0) {
       const int k = (int)std::min<long>(n, kResidentSteps);
       EHD_CK(launch_resident(step_args(r, r->cur), poisson_args(r, true), r->storage, k, r->stream));
+      r->after_on_chip = true;
       n -= k;
       r->step += k;
     }
@@ -1194,11 +1204,13 @@ ehd_status ehd_step(ehd_run* r, long n) {
       if (st != EHD_OK) return st;
     }
     EHD_CK(cudaGraphLaunch(r->graph[r->cur], r->stream));
+    r->after_on_chip = false;
     n -= kGraphSteps;
     r->step += kGraphSteps;
   }
   for (; n > 0; --n) {
     EHD_CK(enqueue_step(r, r->cur, r->step % kGraphSteps));
+    r->after_on_chip = false;
     r->cur = 1 - r->cur;
     r->step += 1;
   }
@@ -1245,6 +1257,7 @@ ehd_status ehd_step_profile(ehd_run* r, long n, double* ms_out) {
     if (e == cudaSuccess && r->pert) e = cudaStreamWaitEvent(r->stream, r->ev_base, 0);
     if (e == cudaSuccess) e = cudaEventRecord(E[3], r->stream);
     if (e == cudaSuccess) {
+      r->after_on_chip = false;
       r->cur = nxt;
       r->step += 1;
     }

@@ -74,12 +74,25 @@ template <class R> struct Cplx { R re, im; };
 
 // ----------------------------------------------------------- kernel args ---
 // Programmatic dependent launch.  A kernel launched with pdl = true may
-// start while the previous kernel of its stream is still running; it must
-// call grid_dep_wait() before touching anything that kernel writes or reads
-// (only tables that no kernel of the step writes may be read before it), and
-// calls grid_dep_launch() after that wait, so that when a kernel starts,
-// every kernel two or more launches back has completed.  Both instructions
-// are no-ops in a kernel launched without the attribute.
+// start while the previous kernel of its stream is still running.  The step's
+// kernels keep these rules:
+//  1. Before grid_dep_wait() a kernel reads nothing that its predecessor
+//     writes, and writes nothing that its predecessor reads or writes.
+//  2. The forward row transforms and the y solves release their successor
+//     (grid_dep_launch, or by ending) only after their own grid_dep_wait().
+//     So when an inverse transform starts, the forward transform and the step
+//     kernel before it have completed, and when a step kernel starts, so have
+//     the solve and all before it.
+//  3. On the strength of 2, and only of 2: the step kernels (k_push, k_march2,
+//     k_step64) read the populations before their wait, and the mean mode's
+//     CTAs of k_irfft_warp read the m = 0 coefficients and the wall-flux
+//     partials without one.  A step kernel is therefore launched with pdl only
+//     where a Poisson solve lies between it and the populations' last writer;
+//     behind k_resident, which is that writer itself, it is not.
+//  4. The step kernels and the mean mode's CTAs may release before their wait:
+//     their successor (the forward transform; the next step kernel) touches
+//     what they write after its own wait only.
+// Both instructions are no-ops in a kernel launched without the attribute.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
