@@ -534,7 +534,6 @@ cudaError_t launch_rhoc(const void* g, long long plane, int storage, int Nx, int
 cudaError_t poisson_set_attributes();
 // warp-per-row real FFTs (FP32 path, Nx = 64 ... 2048)
 bool fftw_supported(int Nx);
-cudaError_t fftw_set_tables();
 cudaError_t launch_rfft_warp(const PoissonArgs& a, cudaStream_t s);
 cudaError_t launch_irfft_warp(const PoissonArgs& a, cudaStream_t s);
 // the forward transform after k_push (rows of 64 to 512)

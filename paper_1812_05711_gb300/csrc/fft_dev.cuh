@@ -1,41 +1,54 @@
 // fft_dev.cuh -- device pieces of the FP32 row transforms, shared by the
 // kernels that transform rows (k_fftw.cu) and the one that keeps a whole run
-// on chip (k_resident.cu).  Each translation unit that includes it has its
-// own copy of the tables and sets them with fft_set_tables().
+// on chip (k_resident.cu).
 #pragma once
-
-#include <cmath>
 
 #include "ehd_dev.cuh"
 
 namespace ehd {
 
-static __constant__ float2 c_w32[32];  // exp(-2 pi i k / 32)
-static __constant__ float2 c_w64[64];  // exp(-2 pi i k / 64)
-// the second one rounded to FP32, in global memory for lane-dependent indices
-static __device__ float2 g_w64[64] = {
-    {1.0f, -0.0f}, {0.99518472f, -0.0980171412f}, {0.980785251f, -0.195090324f},
-    {0.956940353f, -0.290284663f}, {0.923879504f, -0.382683426f}, {0.881921291f, -0.471396744f},
-    {0.831469595f, -0.555570245f}, {0.773010433f, -0.634393275f}, {0.707106769f, -0.707106769f},
-    {0.634393275f, -0.773010433f}, {0.555570245f, -0.831469595f}, {0.471396744f, -0.881921291f},
-    {0.382683426f, -0.923879504f}, {0.290284663f, -0.956940353f}, {0.195090324f, -0.980785251f},
-    {0.0980171412f, -0.99518472f}, {6.12323426e-17f, -1.0f}, {-0.0980171412f, -0.99518472f},
-    {-0.195090324f, -0.980785251f}, {-0.290284663f, -0.956940353f}, {-0.382683426f, -0.923879504f},
-    {-0.471396744f, -0.881921291f}, {-0.555570245f, -0.831469595f}, {-0.634393275f, -0.773010433f},
-    {-0.707106769f, -0.707106769f}, {-0.773010433f, -0.634393275f}, {-0.831469595f, -0.555570245f},
-    {-0.881921291f, -0.471396744f}, {-0.923879504f, -0.382683426f}, {-0.956940353f, -0.290284663f},
-    {-0.980785251f, -0.195090324f}, {-0.99518472f, -0.0980171412f}, {-1.0f, -1.22464685e-16f},
-    {-0.99518472f, 0.0980171412f}, {-0.980785251f, 0.195090324f}, {-0.956940353f, 0.290284663f},
-    {-0.923879504f, 0.382683426f}, {-0.881921291f, 0.471396744f}, {-0.831469595f, 0.555570245f},
-    {-0.773010433f, 0.634393275f}, {-0.707106769f, 0.707106769f}, {-0.634393275f, 0.773010433f},
-    {-0.555570245f, 0.831469595f}, {-0.471396744f, 0.881921291f}, {-0.382683426f, 0.923879504f},
-    {-0.290284663f, 0.956940353f}, {-0.195090324f, 0.980785251f}, {-0.0980171412f, 0.99518472f},
-    {-1.83697015e-16f, 1.0f}, {0.0980171412f, 0.99518472f}, {0.195090324f, 0.980785251f},
-    {0.290284663f, 0.956940353f}, {0.382683426f, 0.923879504f}, {0.471396744f, 0.881921291f},
-    {0.555570245f, 0.831469595f}, {0.634393275f, 0.773010433f}, {0.707106769f, 0.707106769f},
-    {0.773010433f, 0.634393275f}, {0.831469595f, 0.555570245f}, {0.881921291f, 0.471396744f},
-    {0.923879504f, 0.382683426f}, {0.956940353f, 0.290284663f}, {0.980785251f, 0.195090324f},
-    {0.99518472f, 0.0980171412f}};
+// exp(-2 pi i k / 32) and exp(-2 pi i k / 64) rounded to FP32.  The tables are
+// part of the module's image: nothing has to be copied before a kernel that
+// reads them may run.
+#define EHD_W32 \
+  {1.0f, -0.0f}, {0.980785251f, -0.195090324f}, {0.923879504f, -0.382683426f}, {0.831469595f, -0.555570245f}, \
+  {0.707106769f, -0.707106769f}, {0.555570245f, -0.831469595f}, {0.382683426f, -0.923879504f}, \
+  {0.195090324f, -0.980785251f}, {6.12323426e-17f, -1.0f}, {-0.195090324f, -0.980785251f}, \
+  {-0.382683426f, -0.923879504f}, {-0.555570245f, -0.831469595f}, {-0.707106769f, -0.707106769f}, \
+  {-0.831469595f, -0.555570245f}, {-0.923879504f, -0.382683426f}, {-0.980785251f, -0.195090324f}, \
+  {-1.0f, -1.22464685e-16f}, {-0.980785251f, 0.195090324f}, {-0.923879504f, 0.382683426f}, \
+  {-0.831469595f, 0.555570245f}, {-0.707106769f, 0.707106769f}, {-0.555570245f, 0.831469595f}, \
+  {-0.382683426f, 0.923879504f}, {-0.195090324f, 0.980785251f}, {-1.83697015e-16f, 1.0f}, \
+  {0.195090324f, 0.980785251f}, {0.382683426f, 0.923879504f}, {0.555570245f, 0.831469595f}, \
+  {0.707106769f, 0.707106769f}, {0.831469595f, 0.555570245f}, {0.923879504f, 0.382683426f}, \
+  {0.980785251f, 0.195090324f}
+#define EHD_W64 \
+  {1.0f, -0.0f}, {0.99518472f, -0.0980171412f}, {0.980785251f, -0.195090324f}, {0.956940353f, -0.290284663f}, \
+  {0.923879504f, -0.382683426f}, {0.881921291f, -0.471396744f}, {0.831469595f, -0.555570245f}, \
+  {0.773010433f, -0.634393275f}, {0.707106769f, -0.707106769f}, {0.634393275f, -0.773010433f}, \
+  {0.555570245f, -0.831469595f}, {0.471396744f, -0.881921291f}, {0.382683426f, -0.923879504f}, \
+  {0.290284663f, -0.956940353f}, {0.195090324f, -0.980785251f}, {0.0980171412f, -0.99518472f}, \
+  {6.12323426e-17f, -1.0f}, {-0.0980171412f, -0.99518472f}, {-0.195090324f, -0.980785251f}, \
+  {-0.290284663f, -0.956940353f}, {-0.382683426f, -0.923879504f}, {-0.471396744f, -0.881921291f}, \
+  {-0.555570245f, -0.831469595f}, {-0.634393275f, -0.773010433f}, {-0.707106769f, -0.707106769f}, \
+  {-0.773010433f, -0.634393275f}, {-0.831469595f, -0.555570245f}, {-0.881921291f, -0.471396744f}, \
+  {-0.923879504f, -0.382683426f}, {-0.956940353f, -0.290284663f}, {-0.980785251f, -0.195090324f}, \
+  {-0.99518472f, -0.0980171412f}, {-1.0f, -1.22464685e-16f}, {-0.99518472f, 0.0980171412f}, \
+  {-0.980785251f, 0.195090324f}, {-0.956940353f, 0.290284663f}, {-0.923879504f, 0.382683426f}, \
+  {-0.881921291f, 0.471396744f}, {-0.831469595f, 0.555570245f}, {-0.773010433f, 0.634393275f}, \
+  {-0.707106769f, 0.707106769f}, {-0.634393275f, 0.773010433f}, {-0.555570245f, 0.831469595f}, \
+  {-0.471396744f, 0.881921291f}, {-0.382683426f, 0.923879504f}, {-0.290284663f, 0.956940353f}, \
+  {-0.195090324f, 0.980785251f}, {-0.0980171412f, 0.99518472f}, {-1.83697015e-16f, 1.0f}, \
+  {0.0980171412f, 0.99518472f}, {0.195090324f, 0.980785251f}, {0.290284663f, 0.956940353f}, \
+  {0.382683426f, 0.923879504f}, {0.471396744f, 0.881921291f}, {0.555570245f, 0.831469595f}, \
+  {0.634393275f, 0.773010433f}, {0.707106769f, 0.707106769f}, {0.773010433f, 0.634393275f}, \
+  {0.831469595f, 0.555570245f}, {0.881921291f, 0.471396744f}, {0.923879504f, 0.382683426f}, \
+  {0.956940353f, 0.290284663f}, {0.980785251f, 0.195090324f}, {0.99518472f, 0.0980171412f}
+static __constant__ float2 c_w32[32] = {EHD_W32};  // for indices known at compile time
+static __constant__ float2 c_w64[64] = {EHD_W64};
+static __device__ float2 g_w64[64] = {EHD_W64};  // for lane-dependent ones
+#undef EHD_W32
+#undef EHD_W64
 
 __host__ __device__ constexpr int bitrev(int i, int n) {
   int r = 0;
@@ -139,8 +152,8 @@ __device__ __forceinline__ float2 cmf0(float2 a, float2 b) {
 __device__ __forceinline__ float2 cmf1(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -(a.y * b.y)), fmaf(a.y, b.x, a.x * b.y));
 }
-// LIT: the E-point transform by literal factors (fft_lit), for a unit that does
-// not set the tables and owes nobody its bits.
+// LIT: the E-point transform by literal factors (fft_lit), for a kernel that
+// owes no other its bits.
 template <int E>
 __device__ __forceinline__ void fft_lit(float (&re)[E], float (&im)[E]) {
   if constexpr (E == 2) {
@@ -280,16 +293,6 @@ __device__ __forceinline__ float2 entangle(float2 sk, float2 sp, float2 wk) {
   const float2 Dv = make_float2(0.5f * (sk.x - sc.x), 0.5f * (sk.y - sc.y));
   const float2 O = cmf1(Dv, make_float2(wk.x, -wk.y));  // D / W^k
   return make_float2(Ev.x - O.y, -(Ev.y + O.x));      // Re(E + i O), -Im: conjugate
-}
-
-static cudaError_t fft_set_tables() {
-  float2 w32[32], w64[64];
-  const double pi = 3.141592653589793238462643383279502884;
-  for (int k = 0; k < 32; ++k) w32[k] = make_float2((float)std::cos(2 * pi * k / 32), (float)-std::sin(2 * pi * k / 32));
-  for (int k = 0; k < 64; ++k) w64[k] = make_float2((float)std::cos(2 * pi * k / 64), (float)-std::sin(2 * pi * k / 64));
-  cudaError_t e = cudaMemcpyToSymbol(c_w32, w32, sizeof w32);
-  if (e != cudaSuccess) return e;
-  return cudaMemcpyToSymbol(c_w64, w64, sizeof w64);
 }
 
 }  // namespace ehd

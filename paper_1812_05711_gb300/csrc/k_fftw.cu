@@ -766,8 +766,6 @@ cudaError_t launch_batch_irfft(const BatchTables& t, int step, int grid, cudaStr
   return e;
 }
 
-cudaError_t fftw_set_tables() { return fft_set_tables(); }
-
 bool fftw_supported(int Nx) { return Nx >= 64 && Nx <= 2048; }
 
 

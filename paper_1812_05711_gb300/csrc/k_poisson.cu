@@ -1466,8 +1466,7 @@ cudaError_t launch_batch_mean(const BatchTables& t, int step, int grid, cudaStre
 }
 
 cudaError_t poisson_set_attributes() {
-  cudaError_t e = fftw_set_tables();
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   if ((e = allow_max_dynamic_smem(k_batch_modes)) != cudaSuccess) return e;
   if ((e = allow_max_dynamic_smem(k_batch_mean)) != cudaSuccess) return e;
   e = set_attrs_t<double>();

@@ -543,12 +543,13 @@ bool resident_config(int Nx, int Ny, int storage, ResidentKernel* k, size_t* sme
 }  // namespace
 
 // Whether this GPU can hold a run of this size in one cluster; sets the
-// kernel's attributes and this unit's tables on the current device.
+// kernel's attributes on the current device (no copies, no synchronisation:
+// ehd_step asks).
 bool resident_supported(int Nx, int Ny, int storage) {
   ResidentKernel k = nullptr;
   size_t smem = 0;
   if (!resident_config(Nx, Ny, storage, &k, &smem)) return false;
-  return cluster_fits(k, kThreads, smem) && fft_set_tables() == cudaSuccess;
+  return cluster_fits(k, kThreads, smem);
 }
 
 cudaError_t launch_resident(const StepArgs& a, const PoissonArgs& pa, int storage, int steps, cudaStream_t s) {

@@ -55,7 +55,8 @@ def captured(stream, call):
         m = ctypes.c_size_t()
         _ck(cu.cuGraphGetEdges_v2(graph, None, None, None, ctypes.byref(m)))
         a, b, d = (vp * m.value)(), (vp * m.value)(), (_EdgeData * m.value)()
-        _ck(cu.cuGraphGetEdges_v2(graph, a, b, d, ctypes.byref(m)))
+        if m.value:
+            _ck(cu.cuGraphGetEdges_v2(graph, a, b, d, ctypes.byref(m)))
         edges = [(names[a[k]], names[b[k]], d[k].type == PROGRAMMATIC) for k in range(m.value)]
         return [v for v in names.values() if v], edges
     finally:
