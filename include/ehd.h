@@ -192,10 +192,9 @@ ehd_status ehd_step_profile(ehd_run* run, long n, double* ms_out);
  * each is resident and waiting when its predecessor ends: 1 the forward row
  * transform, 2 the wavenumber solve, 4 the inverse transform, 8 the step
  * kernel (march form: it stages its first rows' populations before waiting
- * for phi); the default is 15 up to 3 2^16 nodes and for FP64 compute, 6
- * between 2^19 and 2^21 nodes (4 for rows of 2048) and 7 otherwise (2048 x
- * 1680: 114.1 us per step against 117.0 with none); results are the same for
- * every mask),
+ * for phi); the default depends on the size, the compute type and the y
+ * solve and was measured for each (2048 x 1680: 7, 114.1 us per step against
+ * 117.0 with none); results are the same for every mask),
  * EHD_TUNE_FFT_CTA (FP32 rows
  * of 2048: 1, the default, one CTA of 64 threads per row; 0, one warp per
  * row), EHD_TUNE_Y_SOLVER (the y solve of the wavenumbers m >= 1: 0, the

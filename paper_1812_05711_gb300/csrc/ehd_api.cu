@@ -116,7 +116,8 @@ struct ehd_run {
   int resident = -1;   // small FP32 runs step with the whole state on chip (k_resident.cu): -1 not looked at yet
   bool after_on_chip = false;  // the populations' last writer was k_resident: see step_pdl
   bool tuned = false;  // a launch shape was asked for (ehd_tune): the kernel-per-phase step
-  int pdl = 0;         // programmatic dependent launch between the Poisson kernels (off: see ehd_tune)
+  int pdl = 0;         // programmatic dependent launch of the step's kernels (see default_pdl)
+  bool pdl_set = false;  // by ehd_tune
   int fft_cta = 1;     // rows of 2048: CTA-per-row transforms
   int y_solver = 0;    // y solve of m >= 1: 0 tridiagonal, 1 odd-extension transform
   int NE = 0, nfac = -1, fac[16] = {};  // odd-extension length and radices (nfac < 0: unsupported)
@@ -255,6 +256,38 @@ ehd_status upload(ehd_run* r, void* dst, const void* src, size_t bytes) {
 }
 
 bool push_form(const ehd_run* r);
+// Programmatic dependent launch (mask of EHD_TUNE_PDL) of a run whose mask was
+// not set, as measured per step of the march form (runs that step one node per
+// thread take all four).
+//  - FP64, and FP32 up to 3 2^16 nodes: all four kernels (15; perturbation form
+//    128 x 104: 12.8 us against 13.1 with 7).
+//  - The odd-extension y solve up to 2^21 nodes: that solve and the step kernel
+//    (10; 512 x 416: 28.7 against 32.1 with 7, 1024 x 840: 60.1 / 64.3, 2048 x
+//    400: 57.2 / 59.3, and 62.5 with 4).
+//  - From 2^21: the three Poisson kernels (7; 2048 x 1680: 114.1 against 114.7
+//    with 6, 117.0 with none).
+//  - Between 2^19 and 2^21, rows of 2048: the inverse transform only (4; 2048 x
+//    840: 66.7 against 68.1 with 6, 69.4 with 7).
+//  - There, rows of 1024: the wavenumber solve and the inverse transform, which
+//    carries the mean mode (6; 1024 x 840: 38.1 against 41.2 with 7, 39.6 with
+//    none; perturbation form 40.6 / 42.6 / 43.2); from kTallRows the solve and
+//    the step kernel (10; 1024 x 1160: 49.8 against 52.2 with 6; 1024 x 1500:
+//    61.1 / 63.1, BF16 52.9 / 55.8, spectral E_x 66.6 / 72.8; 1024 x 2040: 83.6 /
+//    85.6; but 1024 x 1130: 57.8 / 51.9).
+//  - Otherwise the three Poisson kernels up to 9 2^16 nodes (7; 512 x 416: 19.6
+//    against 21.0 with 15; 512 x 1100: 30.6 against 33.0 with 6; 256 x 2300: 36.9
+//    / 46.9), and the solve and the inverse transform beyond (6; 512 x 1200: 30.9
+//    against 32.4 with 7; 512 x 1300: 32.9 / 33.7; 256 x 4000: 55.2 / 54.8).
+int default_pdl(const ehd_run* r) {
+  const long long nodes = (long long)r->Nx * r->Ny;
+  if (r->real_f64 || nodes <= (3LL << 16)) return 15;
+  if (nodes >= (1LL << 21)) return 7;
+  if (r->y_solver == 1) return 10;
+  if (nodes <= (1LL << 19)) return 7;
+  if (r->Nx == 2048) return 4;
+  if (r->Nx == 1024) return r->Ny >= kTallRows ? 10 : 6;
+  return nodes <= (9LL << 16) ? 7 : 6;
+}
 // Launch mask of the run's step kernel.  Bit 8, its programmatic launch, is
 // safe only where a Poisson solve lies between the kernel and the populations'
 // last writer: the step kernels read the populations before they wait, because
@@ -825,25 +858,7 @@ ehd_status ehd_create(int Nx, int Ny, double T, double C, double M, double Fe, d
     r->bmom = static_cast<double*>(run_alloc(r, 7 * (size_t)Ny * sizeof(double)));
   }
   r->step_kernel = (o.step_kernel >= 0) ? o.step_kernel : (r->real_f64 && !o.ex_spectral) ? 1 : 0;
-  // programmatic dependent launch (mask of EHD_TUNE_PDL), as measured per step
-  // of the march form (runs that step one node per thread take all four).
-  // FP64, and FP32 up to 3 2^16 nodes: all four kernels (15; perturbation form
-  // 128 x 104: 12.8 us against 13.1 with 7).  Up to 2^19
-  // nodes the three Poisson kernels (7; 512 x 416: 19.6 against 21.0 with 15).
-  // Up to 2^21 the wavenumber solve and the inverse transform, which carries
-  // the mean mode (6; 1024 x 840: 38.1 against 41.2 with 7, 39.6 with none;
-  // perturbation form 40.6 / 42.6 / 43.2), rows of 2048 the inverse only (4;
-  // 2048 x 840: 66.7 against 68.1 with 6).  Beyond, all three again (7; 2048 x
-  // 1680: 114.1 against 114.7 with 6, 117.0 with none)
-  {
-    const long long nodes = (long long)Nx * Ny;
-    if (r->real_f64 || nodes <= (3LL << 16))
-      r->pdl = 15;
-    else if (nodes > (1LL << 19) && nodes < (1LL << 21))
-      r->pdl = Nx == 2048 ? 4 : 6;
-    else
-      r->pdl = 7;
-  }
+  r->pdl = default_pdl(r);
   r->cols_per_lane = 2;
   r->nstrips = march_strips(Nx, r->cols_per_lane);
   r->nxb = (r->step_kernel == 0) ? r->nstrips : step_flux_blocks(Nx, r->real_f64);
@@ -1101,6 +1116,7 @@ ehd_status ehd_tune(ehd_run* r, int param, int value) {
     case EHD_TUNE_PDL:
       if (value < 0 || value > 15) return fail(EHD_EINVAL, "programmatic dependent launch: a mask of 1, 2, 4 and 8");
       r->pdl = value;
+      r->pdl_set = true;
       break;
     case EHD_TUNE_FFT_CTA:
       if (value != 0 && value != 1) return fail(EHD_EINVAL, "CTA-per-row transforms must be 0 or 1");
@@ -1118,6 +1134,7 @@ ehd_status ehd_tune(ehd_run* r, int param, int value) {
           return fail(EHD_EINVAL, "odd-extension column of %d points exceeds shared memory", r->NE);
       }
       r->y_solver = value;
+      if (!r->pdl_set) r->pdl = default_pdl(r);
       break;
     }
     case EHD_TUNE_COLS_PER_LANE:

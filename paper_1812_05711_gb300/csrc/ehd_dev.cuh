@@ -476,6 +476,11 @@ int batch_modes_ctas_per_sm(int smem);
 // perturbation-form members: the FP64 base step and its potential
 cudaError_t launch_batch_base(const BatchTables& t, int step, int max_runs, int max_ny, cudaStream_t s);
 constexpr int kBatchTileModes = 8;
+// From here an SM holds one tile of the wavenumber solve and no longer two (96
+// bytes a row and 5 KB of scratch), and launching the solve ahead of its
+// predecessor's end starts to pay for rows of 1024 (measured on both sides of
+// the line: see default_pdl).
+constexpr int kTallRows = 1140;
 
 
 

@@ -602,8 +602,9 @@ __global__ void __launch_bounds__(128) k_rfft_warp(PoissonArgs a) {
   } else {
     grid_dep_wait();
     // rows of 1024: the wavenumber solve is not released early (see
-    // k_rfft_push; 1024 x 840: 38.1 us per step against 39.2)
-    if constexpr (E > 16) grid_dep_launch();
+    // k_rfft_push; 1024 x 840: 38.1 us per step against 39.2) below kTallRows
+    // (1024 x 1500: 61.1 with the release against 62.9)
+    if (E > 16 || a.Ny >= kTallRows) grid_dep_launch();
     if (y < a.Ny) rfft_warp_rows<E, 1>(a, y, smem[warp]);
   }
 }
