@@ -51,7 +51,14 @@ constexpr double kPi = 3.141592653589793238462643383279502884;
 constexpr int kGraphSteps = 16;  // steps per captured graph (even: buffer parity)
 constexpr int kPushPdl = 15;  // its kernels are all launched programmatically
 constexpr long long kPushNodes = 1LL << 19;  // largest run that steps one node per thread
-constexpr int kResidentSteps = 4096;  // steps per launch of the on-chip form
+// Steps per launch of the on-chip form.  Between launches other streams' kernels
+// get the cluster's 16 SMs, and waiting clusters theirs: beside 8 (16) runs of
+// 128 x 104 a 1024 x 840 run takes 46.1 (43.9) us per step, 44.2 (44.1) when those
+// ran a kernel per phase, but 107 (170) with launches of 4096 steps and 52.7 (47.0)
+// with 512; eight such runs at once take 1.00 us per run and step against 1.58
+// (2.61 with a kernel per phase).  A run alone pays 6.38 for 6.33, 64 x 52 4.37 for
+// 4.33; with 128 steps 6.41.
+constexpr int kResidentSteps = 256;
 constexpr int kSlabShift = 4;    // default slab_shift of large runs (rows per step)
 
 // wall-flux partials per wall, whichever step kernel writes them
