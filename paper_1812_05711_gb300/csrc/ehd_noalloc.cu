@@ -313,20 +313,32 @@ template <int E>
 struct Lay {
   static constexpr int Nx = 64 * E, L = 32 * E, kModes = L / kClusterCtas;
   int rows, spec, col, row, mean, pb;  // float2 offsets
+  // A wavenumber's column: 32 chunks of `chunk` rows (a lane each), an odd
+  // number of float2 apart -- with the rows packed, the lanes of a solve met in
+  // one or two banks whenever the chunk's length was a multiple of 16 or 8 (512
+  // x 512: 48.9 us a call, three kernels 41.2) -- and the columns too.
+  int chunk, chunk_pitch, col_pitch;
   size_t bytes;
   __host__ __device__ explicit Lay(int Ny) {
     rows = (Ny + kClusterCtas - 1) / kClusterCtas;
+    chunk = (Ny + 31) / 32;
+    chunk_pitch = chunk | 1;
+    col_pitch = 32 * chunk_pitch + 1;
     spec = 0;
     col = spec + rows * (L + 2);
-    row = col + kModes * (Ny + 1);
+    row = col + kModes * col_pitch;
     mean = row + kWarps * kLaneRow<E>;
     pb = mean + 2 * Ny;
     bytes = sizeof(float2) * (size_t)(pb + rows);
   }
+  // row y's place in a column; inv = 2^32 / chunk + 1 (y / chunk exactly for y
+  // below 2^25), as a division costs a row 0.3 us
+  __device__ int in_col(int y, unsigned inv) const { return y + (int)__umulhi(y, inv) * (chunk_pitch - chunk); }
 };
+unsigned chunk_inverse(int Ny) { return (unsigned)((1ull << 32) / ((Ny + 31) / 32) + 1); }  // (chunk 1: unused)
 
 template <int E>
-__global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, float ieps, const float* __restrict__ rhoc,
+__global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, unsigned inv, float ieps, const float* __restrict__ rhoc,
                                                        float* __restrict__ phi, Ptrs p, PoissonArgs pa) {
   using La = Lay<E>;
   constexpr int Nx = La::Nx, L = La::L, ML = La::kModes;
@@ -360,7 +372,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, float ieps, const
   // ---- rows: s = -rho_c / eps, its sum (pairs of FP32 numbers, exact), the
   // transform of what differs from the row's first value
   for (int r = warp; r < nr; r += kWarps) {
-    const int y = r0 + r;
+    const int y = r0 + r, yc = la.in_col(y, inv);
     const float2* src = reinterpret_cast<const float2*>(rhoc + (size_t)y * Nx);
     float re[E], im[E];
     float hi = 0.0f, lo = 0.0f;
@@ -391,7 +403,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, float ieps, const
     fft.run(re, im, lane);
     if (lane == 0) {
       st_peer(peer_addr(mean_v + y, kMeanCta), make_float2(hi, lo));
-      st_peer(peer_addr(col + (ML - 1) * (Ny + 1) + y, kClusterCtas - 1), make_float2(2.0f * (re[0] - im[0]), 0.0f));
+      st_peer(peer_addr(col + (ML - 1) * la.col_pitch + yc, kClusterCtas - 1), make_float2(2.0f * (re[0] - im[0]), 0.0f));
     }
     lane_fft_store<E>(re, im, rowbuf, lane);
     // S[k] = E + W^k O from E = Z[k] + Z*[L - k], O = (Z[k] - Z*[L - k]) / i
@@ -403,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, float ieps, const
       const float Er = zk.x + zp.x, Ei = zk.y - zp.y, Dr = zk.x - zp.x, Di = zk.y + zp.y;
       const int m = k - 1;
       if (m >= 0)
-        st_peer(peer_addr(col + (m % ML) * (Ny + 1) + y, m / ML),
+        st_peer(peer_addr(col + (m % ML) * la.col_pitch + yc, m / ML),
                 make_float2(fmaf(wk[j].x, Di, fmaf(wk[j].y, Dr, Er)), fmaf(wk[j].y, Di, fmaf(-wk[j].x, Dr, Ei))));
     }
     __syncwarp();
@@ -427,11 +439,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, float ieps, const
     });
   } else {
     const int nw = rank == kMeanCta ? kMeanWarp : kWarps;
-    const int C = (Ny + 31) >> 5, j0 = min(lane * C, Ny), j1 = min(j0 + C, Ny);
+    const int C = la.chunk, j0 = min(lane * C, Ny), j1 = min(j0 + C, Ny);
     for (int q = warp; q < ML; q += nw) {
       const int m = rank * ML + q + 1;
       const float* __restrict__ r = p.piv + (size_t)m * Ny;
-      float2* d = col + q * (Ny + 1);
+      float2* d = col + q * la.col_pitch + lane * (la.chunk_pitch - C);  // d[j]: row j of this lane's chunk
       float al = 1.0f;
       float2 br = make_float2(0.0f, 0.0f);
       for (int j = j0; j < j1; ++j) {
@@ -514,7 +526,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, float ieps, const
 }
 
 // The cluster kernel of a grid, nullptr where it does not apply.
-using Kernel = void (*)(int, float, const float*, float*, Ptrs, PoissonArgs);
+using Kernel = void (*)(int, unsigned, float, const float*, float*, Ptrs, PoissonArgs);
 Kernel pick(int Nx, int Ny, size_t* smem) {
   if (Ny < kClusterCtas || (long long)Nx * Ny > (1LL << 18)) return nullptr;
   switch (Nx) {
@@ -599,7 +611,7 @@ extern "C" ehd_status ehd_poisson_noalloc(int Nx, int Ny, double eps, double phi
       cudaLaunchAttribute at[1];
       cudaLaunchConfig_t c;
       ehd::cluster_launch_config(&c, at, na::kThreads, smem, s);
-      if (cudaLaunchKernelEx(&c, kernel, Ny, (float)(1.0 / eps), rhoc, phi, p, pa) != cudaSuccess)
+      if (cudaLaunchKernelEx(&c, kernel, Ny, na::chunk_inverse(Ny), (float)(1.0 / eps), rhoc, phi, p, pa) != cudaSuccess)
         return na_fail(EHD_ECUDA, "ehd_poisson_noalloc: kernel launch failed");
       return EHD_OK;
     }
