@@ -297,12 +297,14 @@ __global__ void __launch_bounds__(256) k_na_inv(int Nx, int Ny, float* __restric
 // The whole solve by one cluster of 16 CTAs, for grids whose spectrum fits
 // their shared memory (64 to 512 columns, up to 2^18 nodes).  A small solve is
 // bound by its launches and by the chain of each kernel, not by the work: the
-// three kernels above take 24.6 us a call at 256 x 208 (radix-2 rows with a
-// barrier a stage, an FP64 elimination of the mean mode), of which the data
-// would take 0.1; this one takes 12.3 (64 x 56: 16.4 -> 7.7; 512 x 416: 32.8 ->
-// 26.1, the last size where 16 SMs are enough).  Here a warp transforms a row (LaneFft), the wavenumbers'
-// columns are written into the CTA that solves them and back into the rows'
-// owners, and the mean mode is the FP64 double prefix sum of the run's solver.
+// three kernels above take 24.7 to 26.7 us a call at 256 x 208 (radix-2 rows with
+// a barrier a stage, an FP64 elimination of the mean mode), of which the data
+// would take 0.1; this one takes 12.4 (64 x 56: 16.5 -> 8.3; 512 x 416: 32.9 ->
+// 28.2; 512 x 512: 41 -> 35.6; calls back to back, on one machine -- a call that
+// the caller waits for takes 34 -> 22 us at 256 x 208).  Here a warp transforms a
+// row (LaneFft), the wavenumbers' columns are written into the CTA that solves
+// them and back into the rows' owners, and the mean mode is the FP64 double
+// prefix sum of the run's solver.
 namespace na {
 using namespace ehd;
 constexpr int kThreads = 512, kWarps = kThreads / 32;
@@ -337,8 +339,29 @@ struct Lay {
 };
 unsigned chunk_inverse(int Ny) { return (unsigned)((1ull << 32) / ((Ny + 31) / 32) + 1); }  // (chunk 1: unused)
 
+// A sum as three FP32 numbers a + b + c, the error of each addition carried into
+// the next part (Knuth's two-sum).
+struct Sum3 {
+  float a = 0.0f, b = 0.0f, c = 0.0f;
+  __device__ void add(float v) {
+    float e;
+    two_sum_f(a, v, a, e);
+    two_sum_f(b, e, b, e);
+    c += e;
+  }
+  __device__ void add(float a2, float b2, float c2) {
+    float e, f;
+    two_sum_f(a, a2, a, e);
+    two_sum_f(b, b2, b, f);
+    c += c2 + f;
+    two_sum_f(b, e, b, f);
+    c += f;
+  }
+};
+
+// hieps: 1 / (2 eps)
 template <int E>
-__global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, unsigned inv, float ieps, const float* __restrict__ rhoc,
+__global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, unsigned inv, float hieps, const float* __restrict__ rhoc,
                                                        float* __restrict__ phi, Ptrs p, PoissonArgs pa) {
   using La = Lay<E>;
   constexpr int Nx = La::Nx, L = La::L, ML = La::kModes;
@@ -369,45 +392,45 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, unsigned inv, flo
   for (int j = 0; j < E; ++j) wk[j] = tw[lane + 32 * j];
   cluster_sync();  // every CTA runs: its shared memory may be written
 
-  // ---- rows: s = -rho_c / eps, its sum (pairs of FP32 numbers, exact), the
-  // transform of what differs from the row's first value
+  // ---- rows: half of s = -rho_c / eps, the row's sum, and the transform of what
+  // differs from the row's first value.  The sum is held in three FP32 numbers
+  // whose rounding errors are carried on (FP64 additions, 16 cycles of the SM
+  // each, would be most of a small solve): over values spread across 2^60 it is
+  // within 3e-21 of the largest, an FP64 sum within 9e-16, two FP32 numbers
+  // within 2e-14.  Its terms are s / Nx, so that it is finite where every s is.
   for (int r = warp; r < nr; r += kWarps) {
     const int y = r0 + r, yc = la.in_col(y, inv);
     const float2* src = reinterpret_cast<const float2*>(rhoc + (size_t)y * Nx);
     float re[E], im[E];
-    float hi = 0.0f, lo = 0.0f;
+    Sum3 sum;
 #pragma unroll
     for (int j = 0; j < E; ++j) {
       const float2 v = src[lane + 32 * j];
-      re[j] = -v.x * ieps;
-      im[j] = -v.y * ieps;
+      re[j] = -v.x * hieps;
+      im[j] = -v.y * hieps;
     }
     const float c0 = __shfl_sync(0xffffffffu, re[0], 0);
 #pragma unroll
     for (int j = 0; j < E; ++j) {
-      float e;
-      two_sum_f(hi, re[j], hi, e);
-      lo += e;
-      two_sum_f(hi, im[j], hi, e);
-      lo += e;
+      sum.add(re[j] * (2.0f / Nx));
+      sum.add(im[j] * (2.0f / Nx));
       re[j] -= c0;
       im[j] -= c0;
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      float e;
-      const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-      two_sum_f(hi, h2, hi, e);
-      lo = lo + l2 + e;
-    }
+    for (int o = 16; o > 0; o >>= 1)
+      sum.add(__shfl_xor_sync(0xffffffffu, sum.a, o), __shfl_xor_sync(0xffffffffu, sum.b, o),
+              __shfl_xor_sync(0xffffffffu, sum.c, o));
     fft.run(re, im, lane);
     if (lane == 0) {
-      st_peer(peer_addr(mean_v + y, kMeanCta), make_float2(hi, lo));
+      // (the third part waits in the mean mode's scratch half of the array)
+      st_peer(peer_addr(mean_v + y, kMeanCta), make_float2(sum.a, sum.b));
+      st_peer(peer_addr(mean_v + Ny + y, kMeanCta), make_float2(sum.c, 0.0f));
       st_peer(peer_addr(col + (ML - 1) * la.col_pitch + yc, kClusterCtas - 1), make_float2(2.0f * (re[0] - im[0]), 0.0f));
     }
     lane_fft_store<E>(re, im, rowbuf, lane);
     // S[k] = E + W^k O from E = Z[k] + Z*[L - k], O = (Z[k] - Z*[L - k]) / i
-    // (twice the coefficients: the halves join the inverse's scale)
+    // (the halves are in the values transformed)
 #pragma unroll
     for (int j = 0; j < E; ++j) {
       const int k = lane + 32 * j;
@@ -428,7 +451,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, unsigned inv, flo
     const int t = tid - 32 * kMeanWarp;
     for (int j = t; j < Ny; j += kMeanNT) {
       const float2 v = reinterpret_cast<const float2*>(mean_v)[j];
-      mean_v[j] = (double)v.x + (double)v.y;
+      mean_v[j] = (double)Nx * ((double)v.x + ((double)v.y + (double)reinterpret_cast<const float2*>(mean_v)[Ny + j].x));
     }
     sub_sync<kMeanNT>();
     mean_mode_core<double, kMeanNT>(pa, mean_v, ms, t, [&](int j, double pc, double) {
@@ -495,8 +518,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve(int Ny, unsigned inv, flo
   }
   cluster_sync();
 
-  // ---- rows back: phi = mean + inverse transform, the sum in pairs
-  const float scale = 0.25f / (float)L;  // both halves and 1 / L
+  // ---- rows back: phi = mean + inverse transform.  The FP64 mean as a pair of
+  // FP32 numbers: the sum rounds as the FP64 one (error of 4e6 random sums at
+  // most 0.5 ulp in both, not one different).
+  const float scale = 0.5f / (float)L;  // the halves and 1 / L
   for (int r = warp; r < nr; r += kWarps) {
     const float2* s = spec + r * (L + 2);
     float re[E], im[E];
@@ -611,7 +636,7 @@ extern "C" ehd_status ehd_poisson_noalloc(int Nx, int Ny, double eps, double phi
       cudaLaunchAttribute at[1];
       cudaLaunchConfig_t c;
       ehd::cluster_launch_config(&c, at, na::kThreads, smem, s);
-      if (cudaLaunchKernelEx(&c, kernel, Ny, na::chunk_inverse(Ny), (float)(1.0 / eps), rhoc, phi, p, pa) != cudaSuccess)
+      if (cudaLaunchKernelEx(&c, kernel, Ny, na::chunk_inverse(Ny), 0.5f * (float)(1.0 / eps), rhoc, phi, p, pa) != cudaSuccess)
         return na_fail(EHD_ECUDA, "ehd_poisson_noalloc: kernel launch failed");
       return EHD_OK;
     }
