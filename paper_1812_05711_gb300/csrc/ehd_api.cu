@@ -705,7 +705,7 @@ ehd_status ehd_footprint(int Nx, int Ny, int storage, size_t* bytes) {
       16 * 8 + 64, (size_t)reduce_state_blocks() * 6 * 8,
       (3 * (2 * ny + 2) + (size_t)Nx / 2 + 1) * rs,                          // odd-extension tables
       9 * ny * 8, 9 * ny * 8, 9 * ny * 8, 9 * ny * 8, ny * 8, ny * 8, ny * 8,  // perturbation-form base
-      ny * 16, ny * 16};
+      ny * 16, ny * 16, (6 * ny + 2 * (size_t)base_chunks(Ny)) * 8, 7 * ny * 8};
   size_t b = 0;
   for (size_t v : bufs) {
     const size_t g = (v > (1u << 20)) ? (2u << 20) : 512;
