@@ -92,6 +92,9 @@ template <class R> struct Cplx { R re, im; };
 //  4. The step kernels and the mean mode's CTAs may release before their wait:
 //     their successor (the forward transform; the next step kernel) touches
 //     what they write after its own wait only.
+//  5. What a predecessor may still write while the kernel is resident is read
+//     with plain loads, not through the non-coherent path (__ldg, or a const
+//     __restrict__ pointer), whose data must not change in the kernel's life.
 // Both instructions are no-ops in a kernel launched without the attribute.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }

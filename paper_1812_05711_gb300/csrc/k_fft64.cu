@@ -121,28 +121,27 @@ __global__ void __launch_bounds__(Row64<LG>::kThreads) k_rfft64(PoissonArgs a) {
   double cs = 0.0;
   const long long row = (long long)(live ? y : 0) * a.P;
   if constexpr (FROMG) {
-    const double* __restrict__ g = static_cast<const double*>(a.g) + row;
-    cs = 2.25 * s * __ldg(g);  // near the row's mean: g_0 is about 4/9 rho_c
+    const double* g = static_cast<const double*>(a.g) + row;
+    cs = 2.25 * s * g[0];  // near the row's mean: g_0 is about 4/9 rho_c
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const double2* __restrict__ p = reinterpret_cast<const double2*>(g) + t + q * C::T;
-      double2 r = __ldg(p);
+      const double* p = g + 2 * (t + q * C::T);
+      double2 r = *reinterpret_cast<const double2*>(p);
 #pragma unroll
-      for (int i = 1; i < 9; ++i) r = add64(r, __ldg(reinterpret_cast<const double2*>(
-                                      reinterpret_cast<const double*>(p) + i * a.gplane)));
+      for (int i = 1; i < 9; ++i) r = add64(r, *reinterpret_cast<const double2*>(p + i * a.gplane));
       v[q] = make_double2(fma(r.x, s, -cs), fma(r.y, s, -cs));
     }
   } else {
-    const double* __restrict__ rc = static_cast<const double*>(a.rhoc) + row;
+    const double* rc = static_cast<const double*>(a.rhoc) + row;
     const double *rdn, *rup;
     rhoc_partials<double>(a, live ? y : 0, rdn, rup);
-    cs = s * __ldg(rc);
+    cs = s * rc[0];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int n = t + q * C::T;
-      double2 r = __ldg(reinterpret_cast<const double2*>(rc) + n);
-      if (rdn) r = add64(r, __ldg(reinterpret_cast<const double2*>(rdn) + n));
-      if (rup) r = add64(r, __ldg(reinterpret_cast<const double2*>(rup) + n));
+      double2 r = reinterpret_cast<const double2*>(rc)[n];
+      if (rdn) r = add64(r, reinterpret_cast<const double2*>(rdn)[n]);
+      if (rup) r = add64(r, reinterpret_cast<const double2*>(rup)[n]);
       v[q] = make_double2(fma(r.x, s, -cs), fma(r.y, s, -cs));
     }
   }
@@ -191,7 +190,7 @@ __global__ void __launch_bounds__(Row64<LG>::kThreads) k_irfft64(PoissonArgs a) 
 #pragma unroll
   for (int h = 0; h < 2; ++h) w[h] = __ldg(tw + t + h * C::T);
   grid_dep_wait();
-  const double2* __restrict__ spec = static_cast<const double2*>(a.spec) + (long long)(live ? y : 0) * a.Mp;
+  const double2* spec = static_cast<const double2*>(a.spec) + (long long)(live ? y : 0) * a.Mp;
   auto coef = [&](int k) {
     const double2 c = spec[k];
     if constexpr (!DX) {

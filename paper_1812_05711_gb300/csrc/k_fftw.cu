@@ -388,9 +388,9 @@ __global__ void __launch_bounds__(kCtaT, 12) k_rfft_cta(PoissonArgs a) {
   // A row constant c0 is taken out before the transform: the differences are
   // exact (Sterbenz) and small, so the transform's rounding scales with the
   // row's variation, and only the m = 0 bin depends on c0.
-  float c0 = __ldg(row);
-  if (rdn) c0 += __ldg(rdn);
-  if (rup) c0 += __ldg(rup);
+  float c0 = row[0];
+  if (rdn) c0 += rdn[0];
+  if (rup) c0 += rup[0];
   float re[16], im[16];
 #pragma unroll
   for (int n1 = 0; n1 < 16; ++n1) {
@@ -790,15 +790,15 @@ cudaError_t launch_rfft_warp(const PoissonArgs& a, cudaStream_t s) {
 template <class S>
 __device__ __forceinline__ float2 ld_pair(const S* p) {
   if constexpr (sizeof(S) == 8) {
-    const double2 v = __ldg(reinterpret_cast<const double2*>(p));
+    const double2 v = *reinterpret_cast<const double2*>(p);
     return make_float2((float)v.x, (float)v.y);
   } else if constexpr (sizeof(S) == 4) {
-    return __ldg(reinterpret_cast<const float2*>(p));
+    return *reinterpret_cast<const float2*>(p);
   } else if constexpr (std::is_same_v<S, __half>) {
-    const float2 v = __half22float2(__ldg(reinterpret_cast<const __half2*>(p)));
+    const float2 v = __half22float2(*reinterpret_cast<const __half2*>(p));
     return make_float2(v.x * kHalfUnscale, v.y * kHalfUnscale);
   } else {
-    return __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162*>(p)));
+    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
   }
 }
 
@@ -865,7 +865,7 @@ __global__ void __launch_bounds__(128) k_rfft_push(PoissonArgs a) {
   const float s = live ? __ldg(a.rch + y) : 0.0f;
   grid_dep_wait();
   if (live) {
-    const S* __restrict__ g = static_cast<const S*>(a.g) + (long long)y * a.P;
+    const S* g = static_cast<const S*>(a.g) + (long long)y * a.P;
     const bool first = slab_first(y, a.xslab), last = slab_last(y, a.Ny, a.xslab);
 #pragma unroll
     for (int p = t; p < L; p += T) {

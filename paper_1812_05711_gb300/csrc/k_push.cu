@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(128) k_push(StepArgs a, int log2Nx) {
   const R s_dn = (y > 0) ? (R)__ldg(a.rch + y - 1) : sy;
   grid_dep_wait();  // the populations are the step's before; the potential's kernels end here
   const int xl = (x - 1) & (Nx - 1), xr = (x + 1) & (Nx - 1);
-  const R* __restrict__ ph = static_cast<const R*>(a.dphi) + (long long)y * P;
+  const R* ph = static_cast<const R*>(a.dphi) + (long long)y * P;
   const R gwall = (a.wall_mode == 0) ? R(-1) : R(0);
   const R pc = ph[x];
   const R pm = (y > 0) ? ph[x - P] : gwall * pc;

@@ -247,13 +247,13 @@ __global__ void __launch_bounds__(kStep64Threads, 16) k_step64(StepArgs a, Colli
     const int xl = (x == 0) ? Nx - 1 : x - 1;
     const int xr = (x == Nx - 1) ? 0 : x + 1;
     // E = -grad phi, central differences; phi = phibar(y) + dphi
-    const double* __restrict__ dp = static_cast<const double*>(a.dphi) + c;
+    const double* dp = static_cast<const double*>(a.dphi) + c;
     const double gwall = (a.wall_mode == 0) ? -1.0 : 0.0;
-    const double pW = __ldg(dp - x + xl), pE = __ldg(dp - x + xr);
-    const double pS = (y > 0) ? __ldg(dp - P) : gwall * __ldg(dp);
-    const double pN = (y < Ny - 1) ? __ldg(dp + P) : gwall * __ldg(dp);
+    const double pW = dp[xl - x], pE = dp[xr - x];
+    const double pS = (y > 0) ? dp[-P] : gwall * dp[0];
+    const double pN = (y < Ny - 1) ? dp[P] : gwall * dp[0];
     const double Ex = -0.5 * (pE - pW);
-    const double Ey = fma(-0.5, pN - pS, __ldg(static_cast<const double*>(a.Ebar) + y));
+    const double Ey = fma(-0.5, pN - pS, static_cast<const double*>(a.Ebar)[y]);
     bool bad;
     collide_f64(f, g, Ex, Ey, a.mub, k64, bad);
     if (bad) atomicOr(a.err, 1);
