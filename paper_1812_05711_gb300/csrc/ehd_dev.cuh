@@ -205,13 +205,18 @@ struct StepArgs {
 //   - the rest population takes what the pairs leave of the density, so the
 //     mass and charge of a node are conserved to a rounding that has no
 //     preferred sign, whatever the rounding of the constants;
-//   - 1 / rho by one third-order Householder step x (1 + e + e^2), e = 1 -
-//     rho x, from the hardware's approximation.
+//   - 1 / rho by two Newton-Raphson steps x' = x + x (1 - rho x) from the
+//     hardware's approximation (see recip_f64).
+// 1 / v for 2^-1000 < |v| < 2^1000.  The approximation takes and gives 20
+// mantissa bits, so 1 - v x is below 2^-18; a step squares it, so after the
+// second the truncation is below 2^-72 and the error that of the last rounding:
+// half an ulp and 2^-19 of one, as the correctly rounded division's but for
+// quotients that lie that close to a tie.
 __device__ __forceinline__ double recip_f64(double v) {
   double x;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(v));
-  const double e = fma(-v, x, 1.0);
-  return fma(x, fma(e, e, e), x);
+  x = fma(x, fma(-v, x, 1.0), x);
+  return fma(x, fma(-v, x, 1.0), x);
 }
 // finite: the exponent bits are not all ones (an integer test: an FP64
 // compare would take an FP64 slot)
