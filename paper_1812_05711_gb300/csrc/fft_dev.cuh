@@ -70,8 +70,11 @@ struct FftStage {
       for (int k = 0; k < LEN / 2; ++k) {
         const float2 w = c_w32[k * (32 / LEN)];
         const int u = b * LEN + k, v = u + LEN / 2;
-        const float tr = re[v] * w.x - im[v] * w.y;
-        const float ti = re[v] * w.y + im[v] * w.x;
+        // cmf0, without the multiplications by W^0 = 1 (an eighth to a half of
+        // them: with the rounding stated, 1024 x 840 BF16 35.3 us per step
+        // against 36.0)
+        const float tr = k == 0 ? re[v] : fmaf(re[v], w.x, -(im[v] * w.y));
+        const float ti = k == 0 ? im[v] : fmaf(re[v], w.y, im[v] * w.x);
         // the pair's sum and difference as packed two-float adds
         const float2 a = make_float2(re[u], im[u]);
         const float2 lo = __fadd2_rn(a, make_float2(-tr, -ti)), hi = __fadd2_rn(a, make_float2(tr, ti));
@@ -108,6 +111,14 @@ __device__ __forceinline__ void fft_reg(float (&re)[M], float (&im)[M]) {
 __device__ __forceinline__ float2 cm(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
+// The same product with its rounding stated: which product of the imaginary
+// part is rounded before the fused multiply-add.
+__device__ __forceinline__ float2 cmf0(float2 a, float2 b) {
+  return make_float2(fmaf(a.x, b.x, -(a.y * b.y)), fmaf(a.x, b.y, a.y * b.x));
+}
+__device__ __forceinline__ float2 cmf1(float2 a, float2 b) {
+  return make_float2(fmaf(a.x, b.x, -(a.y * b.y)), fmaf(a.y, b.x, a.x * b.y));
+}
 
 __device__ __forceinline__ void two_sum_f(float a, float b, float& s, float& e) {
   s = a + b;
@@ -124,7 +135,7 @@ __device__ __forceinline__ void four_step_twiddles(const float2* __restrict__ tw
   float2 c = make_float2(1.0f, 0.0f);
 #pragma unroll
   for (int k2 = 0; k2 < E; ++k2) {
-    if (k2 > 0) c = ((k2 & 3) == 0) ? tw[(2 * lane * k2) & (N - 1)] : cm(c, base);
+    if (k2 > 0) c = ((k2 & 3) == 0) ? tw[(2 * lane * k2) & (N - 1)] : k2 == 1 ? base : cmf0(c, base);
     w[k2] = c;
   }
 }
@@ -141,17 +152,11 @@ __device__ __forceinline__ void four_step_twiddles(const float2* __restrict__ tw
 // repeated them: for E = 2 a warp issued 640 instructions where 110 do.)
 // On return (re[k2], im[k2]) of a lane is X[k2 + E bitrev(lane)].
 //
-// Every product sum below is written with its fused multiply-add, so that the
-// kernels which share this code give a row the same bits whatever surrounds
-// it, and with the one that the compiler forms in the batch's wide transforms
-// (rfft_warp_rows, irfft_warp_rows), so that a run gives the bits it gives in a
-// batch.  The two differ in which product of the imaginary part is rounded.
-__device__ __forceinline__ float2 cmf0(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, -(a.y * b.y)), fmaf(a.x, b.y, a.y * b.x));
-}
-__device__ __forceinline__ float2 cmf1(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, -(a.y * b.y)), fmaf(a.y, b.x, a.x * b.y));
-}
+// Every product sum here and in the wide transforms (rfft_warp_rows,
+// irfft_warp_rows in k_fftw.cu) is written with its fused multiply-add, so that
+// a row has the same bits in every kernel that transforms it: the step of one
+// node per thread sends rows of 1024 through LaneFft, the march form and the
+// batch through the wide form.
 // LIT: the E-point transform by literal factors (fft_lit), for a kernel that
 // owes no other its bits.
 template <int E>

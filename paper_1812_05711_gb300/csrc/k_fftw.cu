@@ -33,7 +33,7 @@ __device__ __forceinline__ void four_step_first(float (&re)[E], float (&im)[E], 
                                                 int r, int lane) {
   fft_reg<E>(re, im);
 #pragma unroll
-  for (int k2 = 0; k2 < E; ++k2) sm[(r * E + k2) * 33 + lane] = cm(make_float2(re[k2], im[k2]), w[k2]);
+  for (int k2 = 0; k2 < E; ++k2) sm[(r * E + k2) * 33 + lane] = cmf1(make_float2(re[k2], im[k2]), w[k2]);
 }
 
 // RE = R E rows of the buffer are written; lanes above them repeat a row (and
@@ -139,8 +139,9 @@ __device__ __forceinline__ void rfft_warp_rows(const PoissonArgs& a, int y0, flo
     const float2 Ev = make_float2(0.5f * (zk.x + zc.x), 0.5f * (zk.y + zc.y));
     const float2 Dv = make_float2(0.5f * (zk.x - zc.x), 0.5f * (zk.y - zc.y));
     const float2 O = make_float2(Dv.y, -Dv.x);
-    const float2 wk = cm(wk2, c_w64[k1]);  // W_N^(k2 + E k1) = W_N^k2 W_64^k1
-    const float2 Sk = make_float2(Ev.x + (wk.x * O.x - wk.y * O.y), Ev.y + (wk.x * O.y + wk.y * O.x));
+    const float2 wk = cmf1(wk2, c_w64[k1]);  // W_N^(k2 + E k1) = W_N^k2 W_64^k1
+    const float2 wO = cmf0(wk, O);
+    const float2 Sk = make_float2(Ev.x + wO.x, Ev.y + wO.y);
     const int k = k2 + E * k1;
     if (live) spec[k] = (k == 0) ? make_float2(0.0f, 0.0f) : Sk;
   }
@@ -176,7 +177,7 @@ __device__ __forceinline__ void irfft_warp_rows(const PoissonArgs& a, int y0, fl
   const float2 wl = tw[lane];
   float2 wk[E];
 #pragma unroll
-  for (int n2 = 0; n2 < E; ++n2) wk[n2] = cm(wl, tw[32 * n2]);
+  for (int n2 = 0; n2 < E; ++n2) wk[n2] = cmf1(wl, tw[32 * n2]);
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int y = y0 + r;
@@ -193,9 +194,9 @@ __device__ __forceinline__ void irfft_warp_rows(const PoissonArgs& a, int y0, fl
       const float2 sc = make_float2(sp.x, -sp.y);
       const float2 Ev = make_float2(0.5f * (sk.x + sc.x), 0.5f * (sk.y + sc.y));
       const float2 Dv = make_float2(0.5f * (sk.x - sc.x), 0.5f * (sk.y - sc.y));
-      const float2 O = cm(Dv, make_float2(wk[n2].x, -wk[n2].y));  // D / W^k
-      re[n2] = Ev.x - O.y;                                        // Re(E + i O)
-      im[n2] = -(Ev.y + O.x);                                     // -Im: conjugate
+      const float2 O = cmf1(Dv, make_float2(wk[n2].x, -wk[n2].y));  // D / W^k
+      re[n2] = Ev.x - O.y;                                          // Re(E + i O)
+      im[n2] = -(Ev.y + O.x);                                       // -Im: conjugate
     }
     four_step_first<E>(re, im, w, sm, r, lane);
   }
@@ -502,9 +503,9 @@ __global__ void __launch_bounds__(kCtaT, 12) k_irfft_cta(PoissonArgs a) {
       dphi2[k1 + 16 * (4 * q + i) + 256 * d] = make_float2(zr[4 * d + i] * inL, -zi[4 * d + i] * inL);
 }
 
-// The same transforms of one row with all lanes at work (LaneFft): the single
-// run's rows of up to 512 reals, bound by the length of one warp's instruction
-// chain.  The same bits as rfft_warp_rows / irfft_warp_rows.
+// The same transforms of one row with all lanes at work (LaneFft): rows of up
+// to 512 reals, and of 1024 after k_push, bound by the length of one warp's
+// instruction chain.  The same bits as rfft_warp_rows / irfft_warp_rows.
 template <int E>
 __device__ __forceinline__ void rfft_lane_charge(const PoissonArgs& a, int y, const float2 (&v)[E],
                                                  const LaneFft<E>& fft, const float2 (&wk)[E], float2* sm) {

@@ -28,6 +28,7 @@
 #include <cooperative_groups.h>
 
 #include "mean_dev.cuh"
+#include "sweep_dev.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -354,7 +355,7 @@ __device__ __forceinline__ void chunk_carries(TileScratch<R, MB, NT>& ts) {
     const R a2 = __shfl_up_sync(0xffffffffu, al, o);
     const R b2r = __shfl_up_sync(0xffffffffu, br.re, o), b2i = __shfl_up_sync(0xffffffffu, br.im, o);
     if (lane >= o) {  // the earlier maps first: x -> al (a2 x + b2) + br
-      br = {al * b2r + br.re, al * b2i + br.im};
+      br = {map_apply(al, b2r, br.re), map_apply(al, b2i, br.im)};
       al = al * a2;
     }
   }
@@ -374,10 +375,10 @@ __device__ __forceinline__ void chunk_carries(TileScratch<R, MB, NT>& ts) {
     for (int k = 0; k < seg; ++k) {
       const R ak = ts.wa[mo][k];
       const Cplx<R> bk = ts.wb[mo][k];
-      vin = {ak * vin.re + bk.re, ak * vin.im + bk.im};
+      vin = {map_apply(ak, vin.re, bk.re), map_apply(ak, vin.im, bk.im)};
     }
   }
-  ts.carry[c][mo] = {ea * vin.re + eb.re, ea * vin.im + eb.im};
+  ts.carry[c][mo] = {map_apply(ea, vin.re, eb.re), map_apply(ea, vin.im, eb.im)};
 }
 
 // One CTA solves wavenumbers m0 .. m0 + MB - 1 of run a (smem_raw: tile
@@ -443,20 +444,24 @@ __device__ __forceinline__ void modes_tile_sweeps(const PoissonArgs& a, int m0, 
   // forward: compose chunk map
   R al = R(1);
   Cplx<R> br = {R(0), R(0)};
-  for (int j = j0; j < j1; ++j) {
-    const R r = rt[j * MB + mo];
-    const Cplx<R> dj = d[j * MB + mo];
-    al = -r * al;
-    if constexpr (sizeof(R) == 8) {
+  if constexpr (sizeof(R) == 8) {
+    for (int j = j0; j < j1; ++j) {
+      const R r = rt[j * MB + mo];
+      const Cplx<R> dj = d[j * MB + mo];
+      al = -r * al;
       // FP64 issue is what bounds these sweeps: r d is formed once and kept,
       // each sweep is then one fused multiply-add per part (12 FP64
       // instructions per value instead of 14)
       const Cplx<R> rd = {r * dj.re, r * dj.im};
       d[j * MB + mo] = rd;
       br = {fma(-r, br.re, rd.re), fma(-r, br.im, rd.im)};
-    } else {
-      br = {r * (dj.re - br.re), r * (dj.im - br.im)};
     }
+  } else {
+    const R* rp = rt + j0 * MB + mo;
+    const Cplx<R>* dp = d + j0 * MB + mo;
+    const ChunkMap cm = chunk_map(j1 - j0, [&](int k) { return rp[k * MB]; }, [&](int k) { return dp[k * MB]; });
+    al = cm.al;
+    br = {cm.br.x, cm.br.y};
   }
   s_al[ch][mo] = al;
   s_br[ch][mo] = br;
@@ -467,15 +472,17 @@ __device__ __forceinline__ void modes_tile_sweeps(const PoissonArgs& a, int m0, 
   Cplx<R> x = s_carry[ch][mo];
   R ab = R(1);
   Cplx<R> bb = {R(0), R(0)};
+  // (unrolled by eight rows: 2048 x 300 31.0 us per step against 31.5)
+#pragma unroll 8
   for (int j = j0; j < j1; ++j) {
     const R r = rt[j * MB + mo];
     const Cplx<R> dj = d[j * MB + mo];
     if constexpr (sizeof(R) == 8)
       x = {fma(-r, x.re, dj.re), fma(-r, x.im, dj.im)};
     else
-      x = {r * (dj.re - x.re), r * (dj.im - x.im)};
+      x = {sweep_value(r, dj.re, x.re), sweep_value(r, dj.im, x.im)};
     d[j * MB + mo] = x;
-    bb = {bb.re + ab * x.re, bb.im + ab * x.im};
+    bb = {map_apply(ab, x.re, bb.re), map_apply(ab, x.im, bb.im)};
     ab = -ab * r;
   }
   tile_sync<NT>();
@@ -494,7 +501,7 @@ __device__ __forceinline__ void modes_tile_sweeps(const PoissonArgs& a, int m0, 
   for (int j = j1 - 1; j >= j0; --j) {
     const R r = rt[j * MB + mo];
     const Cplx<R> dj = d[j * MB + mo];
-    x = {dj.re - r * x.re, dj.im - r * x.im};
+    x = {sweep_back(r, dj.re, x.re), sweep_back(r, dj.im, x.im)};
     if (put) col[(long long)j * Mp] = x;
   }
 }
@@ -666,18 +673,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTileThreads) k_mode
   const bool own = (ch / HALF) == rank;
   const int j0 = min(ch * C, Ny), j1 = min(j0 + C, Ny);
   if (own) {
-    R al = R(1);
-    Cplx<R> br = {R(0), R(0)};
-    for (int j = j0; j < j1; ++j) {
-      const R r = rt[(j - R0) * MB + mo];
-      const Cplx<R> dj = d[(j - R0) * MB + mo];
-      al = -r * al;
-      br = {r * (dj.re - br.re), r * (dj.im - br.im)};
-    }
-    ts.al[ch][mo] = al;
-    ts.br[ch][mo] = br;
-    peer->al[ch][mo] = al;
-    peer->br[ch][mo] = br;
+    const ChunkMap cm = chunk_map(j1 - j0, [&](int k) { return rt[(j0 - R0 + k) * MB + mo]; },
+                                  [&](int k) { return d[(j0 - R0 + k) * MB + mo]; });
+    ts.al[ch][mo] = cm.al;
+    ts.br[ch][mo] = {cm.br.x, cm.br.y};
+    peer->al[ch][mo] = cm.al;
+    peer->br[ch][mo] = {cm.br.x, cm.br.y};
   }
   cl.sync();
   chunk_carries<R, MB, NT, false>(ts);
@@ -689,9 +690,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTileThreads) k_mode
     for (int j = j0; j < j1; ++j) {
       const R r = rt[(j - R0) * MB + mo];
       const Cplx<R> dj = d[(j - R0) * MB + mo];
-      x = {r * (dj.re - x.re), r * (dj.im - x.im)};
+      x = {sweep_value(r, dj.re, x.re), sweep_value(r, dj.im, x.im)};
       d[(j - R0) * MB + mo] = x;
-      bb = {bb.re + ab * x.re, bb.im + ab * x.im};
+      bb = {map_apply(ab, x.re, bb.re), map_apply(ab, x.im, bb.im)};
       ab = -ab * r;
     }
   }
@@ -710,7 +711,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTileThreads) k_mode
     for (int j = j1 - 1; j >= j0; --j) {
       const R r = rt[(j - R0) * MB + mo];
       const Cplx<R> dj = d[(j - R0) * MB + mo];
-      x = {dj.re - r * x.re, dj.im - r * x.im};
+      x = {sweep_back(r, dj.re, x.re), sweep_back(r, dj.im, x.im)};
       d[(j - R0) * MB + mo] = x;
     }
   }

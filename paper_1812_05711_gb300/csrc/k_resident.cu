@@ -33,6 +33,7 @@
 #include "fft_dev.cuh"
 #include "march_dev.cuh"
 #include "mean_dev.cuh"
+#include "sweep_dev.cuh"
 
 namespace ehd {
 
@@ -403,29 +404,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(StepArgs a, PoissonArg
         const float2* c = col + warp * (lay.col_row / 2) + j0;
 #pragma unroll
         for (int k = 0; k < kChunkRows; ++k) d[k] = k < nj ? c[k] : make_float2(0.0f, 0.0f);
-        // forward sweep: the chunk's affine map, the scan over chunks, values.
-        // The map's differences d - r' (..) are fused multiply-adds where the
-        // tile kernels' compiled loop has them (rows of a group of four, the
-        // second of two or three left over), so that the bits are theirs.
-        float al = 1.0f, rp = 0.0f;
-        float2 br = make_float2(0.0f, 0.0f), df = br;
+        // forward sweep: the chunk's affine map, the scan over chunks, values
+        ChunkMap cm;
 #pragma unroll
         for (int k = 0; k < kChunkRows; ++k)
-          if (k < nj) {
-            const float r = piv[k];
-            al = -r * al;
-            const bool fused = k == 1 || (k > 1 && nj == 4);
-            df = fused ? make_float2(fmaf(-rp, df.x, d[k].x), fmaf(-rp, df.y, d[k].y))
-                       : make_float2(__fsub_rn(d[k].x, br.x), __fsub_rn(d[k].y, br.y));
-            br = make_float2(__fmul_rn(r, df.x), __fmul_rn(r, df.y));
-            rp = r;
-          }
+          if (k < nj) cm.row(piv[k], d[k].x, d[k].y, tail_row_fused(k, nj));
+        float al = cm.al;
+        float2 br = cm.br;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
           const float a2 = __shfl_up_sync(0xffffffffu, al, o);
           const float bx = __shfl_up_sync(0xffffffffu, br.x, o), by = __shfl_up_sync(0xffffffffu, br.y, o);
           if (lane >= o) {
-            br = make_float2(fmaf(al, bx, br.x), fmaf(al, by, br.y));
+            br = make_float2(map_apply(al, bx, br.x), map_apply(al, by, br.y));
             al = al * a2;
           }
         }
@@ -437,9 +428,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(StepArgs a, PoissonArg
         for (int k = 0; k < kChunkRows; ++k)
           if (k < nj) {
             const float r = piv[k];
-            x = make_float2(__fmul_rn(r, __fsub_rn(d[k].x, x.x)), __fmul_rn(r, __fsub_rn(d[k].y, x.y)));
+            x = make_float2(sweep_value(r, d[k].x, x.x), sweep_value(r, d[k].y, x.y));
             d[k] = x;
-            br = make_float2(fmaf(al, x.x, br.x), fmaf(al, x.y, br.y));
+            br = make_float2(map_apply(al, x.x, br.x), map_apply(al, x.y, br.y));
             al = -al * r;
           }
         // backward sweep, from the last chunk down
@@ -448,7 +439,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(StepArgs a, PoissonArg
           const float a2 = __shfl_down_sync(0xffffffffu, al, o);
           const float bx = __shfl_down_sync(0xffffffffu, br.x, o), by = __shfl_down_sync(0xffffffffu, br.y, o);
           if (lane + o < 32) {
-            br = make_float2(fmaf(al, bx, br.x), fmaf(al, by, br.y));
+            br = make_float2(map_apply(al, bx, br.x), map_apply(al, by, br.y));
             al = al * a2;
           }
         }
@@ -458,7 +449,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(StepArgs a, PoissonArg
         for (int k = kChunkRows - 1; k >= 0; --k)
           if (k < nj) {
             const float r = piv[k];
-            x = make_float2(fmaf(-r, x.x, d[k].x), fmaf(-r, x.y, d[k].y));
+            x = make_float2(sweep_back(r, d[k].x, x.x), sweep_back(r, d[k].y, x.y));
             st_peer(home[k], x);
           }
       }
