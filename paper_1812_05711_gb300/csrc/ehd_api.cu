@@ -108,6 +108,7 @@ struct ehd_run {
   double* small = nullptr;  // [0] q_in sum, [1] q_out sum, [2..7] last reduction, [8..9] base q_in, q_out
   int* err = nullptr;
   double* red_part = nullptr;
+  int sms = 152;
   int rows = 1;        // rows per CTA of the node-parallel step kernel
   int step_kernel = 0; // 0 march form, 1 node-parallel push form
   int slab_rows = 4;   // rows per warp slab of the march form
@@ -380,7 +381,9 @@ PoissonArgs poisson_args(const ehd_run* r, bool with_flux) {
   a.flux_part = with_flux ? r->flux_part : nullptr;
   a.nflux = r->nxb;
   a.flux_acc = r->small;
-  a.tile_modes = r->tile_modes;
+  // FP64: one warp per wavenumber while there are no more of them than SMs (see
+  // launch_modes64), else two
+  a.tile_modes = (r->tile_modes == 0 && r->real_f64) ? (r->Mh > r->sms ? 2 : 1) : r->tile_modes;
   a.tile_threads = r->tile_threads;
   a.tile_cluster = r->tile_cluster;
   a.tile_tma = r->tile_tma;
@@ -901,10 +904,9 @@ ehd_status ehd_create(int Nx, int Ny, double T, double C, double M, double Fe, d
   // march slabs: as many warps as the GPU holds at once (one wave), at
   // least 4 rows each
   {
-    int sms = 152;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, r->device);
+    cudaDeviceGetAttribute(&r->sms, cudaDevAttrMultiProcessorCount, r->device);
     const long long resident =
-        (long long)sms * march_warps_per_sm(r->storage, r->real_f64, r->cols_per_lane, r->ring_depth);
+        (long long)r->sms * march_warps_per_sm(r->storage, r->real_f64, r->cols_per_lane, r->ring_depth);
     long long rows = ((long long)Ny * r->nstrips + resident - 1) / resident;
     r->slab_rows = (int)std::max(4LL, std::min((long long)Ny, rows));
     // populations larger than L2: the slab partition advances a step, so that

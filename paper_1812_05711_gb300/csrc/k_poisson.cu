@@ -1257,7 +1257,7 @@ cudaError_t modes64_n(const PoissonArgs& a, cudaStream_t s) {
 }
 cudaError_t launch_modes64(const PoissonArgs& a, cudaStream_t s) {
   const int fit = tile_modes(a.Ny, sizeof(Cplx<double>), sizeof(double));
-  switch (std::min(fit, a.tile_modes > 0 ? a.tile_modes : (a.Mh > 152 ? 2 : 1))) {
+  switch (std::min(fit, std::max(1, a.tile_modes))) {
     case 8: return modes64_n<8>(a, s);
     case 4: return modes64_n<4>(a, s);
     case 2: return modes64_n<2>(a, s);
