@@ -36,9 +36,11 @@ import workloads as wl  # noqa: E402
 
 METRIC = "coupled-step GLUPS"
 UNIT = "GLUPS"
-# kernels per coupled step: collide-stream (march form, writes the charge),
-# forward row FFT, mean mode (side stream), wavenumber systems, inverse row FFT
-LAUNCHES_PER_STEP = 5
+# kernels per coupled step of the 2048 x 1680 channel: collide-stream, forward
+# row FFT, mean mode (side stream), wavenumber systems, inverse row FFT; FP64 has
+# the mean mode in the wavenumber systems' launch, as a batch of up to 1024 rows
+LAUNCHES_PER_STEP = {"f32": 5, "bf16": 5, "f16": 5, "f64": 4}
+BATCH_LAUNCHES_PER_STEP = 4
 # algorithmic bytes per node of the fused collide-stream kernel: 9 f + 9 g
 # loaded, 9 f + 9 g stored, one potential value loaded, one charge density
 # stored (both in the compute precision: FP64 for f64 storage, else FP32)
@@ -48,17 +50,33 @@ K4_BYTES_PER_NODE = {"f32": 36 * 4 + 8, "f64": 36 * 8 + 16, "bf16": 36 * 2 + 8, 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of
 # the fused step kernel, from an ncu capture of the 2048 x 1680 FP32 channel
 # in the steady state of this bench (no cache flush between launches: the
-# mean of three consecutive launches); keyed by a hash of the kernel's sources
-# so that it reads null once the kernel has changed since the capture.
+# mean of three consecutive launches); keyed by a hash of the kernel's sources,
+# the headers it includes among them, so that it reads null once the kernel has
+# changed since the capture.
 NCU_TRAFFIC = {("f32", "b117d667c207899e"): (245.364736e6 + 241.394688e6 + 241.035008e6) / 3
                + (262.903808e6 + 260.883456e6 + 260.696832e6) / 3}
 
 
-def _kernel_hash():
+CSRC = os.path.join(ROOT, "paper_1812_05711_gb300", "csrc")
+
+
+def _kernel_sources(csrc=CSRC, name="k_march.cu"):
+    """The source of the fused step kernel and the headers it includes from csrc, in order."""
+    import re
+    found = [name]
+    for f in found:
+        with open(os.path.join(csrc, f)) as fh:
+            for inc in re.findall(r'^#include "([^"]+)"', fh.read(), re.M):
+                if inc not in found and os.path.exists(os.path.join(csrc, inc)):
+                    found.append(inc)
+    return found
+
+
+def _kernel_hash(csrc=CSRC):
     import hashlib
     h = hashlib.sha256()
-    for name in ("k_march.cu", "ehd_dev.cuh"):
-        with open(os.path.join(ROOT, "paper_1812_05711_gb300", "csrc", name), "rb") as fh:
+    for name in _kernel_sources(csrc):
+        with open(os.path.join(csrc, name), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
@@ -349,7 +367,7 @@ def run_ours(args):
                      "whole_step": {"bytes_per_node": K4_BYTES_PER_NODE[storage] + 8, "achieved": step_achieved,
                                     "frac": step_achieved / peak}},
         "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
-        "gpu_launches": (LAUNCHES_PER_STEP + 2 * pert) * args.steps,
+        "gpu_launches": (LAUNCHES_PER_STEP[storage] + 2 * pert) * args.steps,
         "cpu_baseline": cpu,
         "clocks": clocks,
         "check": {"mass": diag["mass"], "charge": diag["charge"], "max_u": diag["max_u"]},
@@ -444,7 +462,7 @@ def run_batch(args):
             "roofline": None,
             "e2e": {"value": cells * K / e2e_s / 1e9, "unit": UNIT, "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h},
-            "gpu_launches": 5 * ticks * args.tick, "cpu_baseline": cpu}
+            "gpu_launches": BATCH_LAUNCHES_PER_STEP * ticks * args.tick, "cpu_baseline": cpu}
     print(json.dumps(line), flush=True)
     batch.close()
     return 0
