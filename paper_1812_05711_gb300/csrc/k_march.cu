@@ -700,12 +700,7 @@ __device__ __forceinline__ void march2_body(const StepArgs& a, int strip, int sl
           n5 = -g7c[j] + R(2) * W2 * rho0 * (R(4.5) * (dx + dy) * (sx + sy2) - w15);
           n6 = -g8c[j] + R(2) * W2 * rho0 * (R(4.5) * (dy - dx) * (sy2 - sx) - w15);
         } else {
-          const R wx = mub * Exs[j], wy = mub * Eys[j];
-          const R w15 = R(1.5) * (wx * wx + wy * wy);
-          const R c2 = wy, c5 = wx + wy, c6 = wy - wx;
-          n2 = -(g4c[j] + R(2) * W1 * sy) + R(2) * W1 * rho0 * (R(1) + R(4.5) * c2 * c2 - w15);
-          n5 = -(g7c[j] + R(2) * W2 * sy) + R(2) * W2 * rho0 * (R(1) + R(4.5) * c5 * c5 - w15);
-          n6 = -(g8c[j] + R(2) * W2 * sy) + R(2) * W2 * rho0 * (R(1) + R(4.5) * c6 * c6 - w15);
+          inject<R>(g4c[j], g7c[j], g8c[j], Exs[j], Eys[j], sy, mub, rho0, n2, n5, n6);
         }
         Uc[0][j] = f4c[j] - wd1;
         Uc[1][j] = f7c[j] - wd2;
@@ -884,8 +879,11 @@ __device__ __forceinline__ void march2_body(const StepArgs& a, int strip, int sl
   }
 }
 
+// FP64 storage: the rows staged leave room for two CTAs per SM, so that bound
+// gives a thread 216 registers instead of 168 (1024 x 840 FP64 storage, FP32
+// compute: 82.9 us per step against 91.0).
 template <class S, class R, int NSTAGE, bool SPECX = false, bool PERT = false>
-__global__ void __launch_bounds__(128) k_march2(StepArgs a) {
+__global__ void __launch_bounds__(128, sizeof(S) == 8 ? 2 : 0) k_march2(StepArgs a) {
   extern __shared__ __align__(16) unsigned char march_smem[];
   // the forward transform (launched with programmatic dependent launch) may
   // become resident as this one-wave grid's CTAs finish; it waits for the
@@ -1234,12 +1232,8 @@ __device__ __forceinline__ void march_tma_body(const StepArgs& a, const MarchTma
       const R Exs[2] = {Ex0, Ex1}, Eys[2] = {Ey0, Ey1};
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        const R wx = mub * Exs[j], wy = mub * Eys[j];
-        const R w15 = R(1.5) * (wx * wx + wy * wy);
-        const R c2 = wy, c5 = wx + wy, c6 = wy - wx;
-        const R n2 = -(g4c[j] + R(2) * W1 * sy) + R(2) * W1 * rho0 * (R(1) + R(4.5) * c2 * c2 - w15);
-        const R n5 = -(g7c[j] + R(2) * W2 * sy) + R(2) * W2 * rho0 * (R(1) + R(4.5) * c5 * c5 - w15);
-        const R n6 = -(g8c[j] + R(2) * W2 * sy) + R(2) * W2 * rho0 * (R(1) + R(4.5) * c6 * c6 - w15);
+        R n2, n5, n6;
+        inject<R>(g4c[j], g7c[j], g8c[j], Exs[j], Eys[j], sy, mub, rho0, n2, n5, n6);
         Uc[0][j] = f4c[j] - wd1;
         Uc[1][j] = f7c[j] - wd2;
         Uc[2][j] = f8c[j] - wd2;

@@ -103,12 +103,8 @@ __global__ void __launch_bounds__(128) k_push(StepArgs a, int log2Nx) {
     put(e + 8 * pl + xr, g[8] + W2 * sh);
   } else {
     // injector: bounce-back of f, anti-bounce-back of g
-    const R wx = mub * Ex, wy = mub * Ey;
-    const R w15 = R(1.5) * (wx * wx + wy * wy);
-    const R c2 = wy, c5 = wx + wy, c6 = wy - wx;
-    const R n2 = -(g[4] + R(2) * W1 * sy) + R(2) * W1 * rho0 * (R(1) + R(4.5) * c2 * c2 - w15);
-    const R n5 = -(g[7] + R(2) * W2 * sy) + R(2) * W2 * rho0 * (R(1) + R(4.5) * c5 * c5 - w15);
-    const R n6 = -(g[8] + R(2) * W2 * sy) + R(2) * W2 * rho0 * (R(1) + R(4.5) * c6 * c6 - w15);
+    R n2, n5, n6;
+    inject<R>(g[4], g[7], g[8], Ex, Ey, sy, mub, rho0, n2, n5, n6);
     put(fo + 2 * pl + x, f[4] - wd1);
     put(fo + 5 * pl + x, f[7] - wd2);
     put(fo + 6 * pl + x, f[8] - wd2);

@@ -298,12 +298,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_resident(StepArgs a, PoissonArg
         }
       } else {
         // injector: bounce-back of f, anti-bounce-back of g
-        const float wx = mub * Ex, wy = mub * Ey;
-        const float w15 = 1.5f * (wx * wx + wy * wy);
-        const float c2 = wy, c5 = wx + wy, c6 = wy - wx;
-        const float n2 = -(g[4] + 2.0f * W1 * sy) + 2.0f * W1 * rho0 * (1.0f + 4.5f * c2 * c2 - w15);
-        const float n5 = -(g[7] + 2.0f * W2 * sy) + 2.0f * W2 * rho0 * (1.0f + 4.5f * c5 * c5 - w15);
-        const float n6 = -(g[8] + 2.0f * W2 * sy) + 2.0f * W2 * rho0 * (1.0f + 4.5f * c6 * c6 - w15);
+        float n2, n5, n6;
+        inject<float>(g[4], g[7], g[8], Ex, Ey, sy, mub, rho0, n2, n5, n6);
         float* d = q + rowb;
         d[2 * RN + x] = rt(f[4] - wd1);
         d[5 * RN + x] = rt(f[7] - wd2);
