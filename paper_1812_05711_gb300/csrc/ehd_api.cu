@@ -268,7 +268,11 @@ bool push_form(const ehd_run* r);
 // not set, as measured per step of the march form (runs that step one node per
 // thread take all four).
 //  - FP64, and FP32 up to 3 2^16 nodes: all four kernels (15; perturbation form
-//    128 x 104: 12.8 us against 13.1 with 7).
+//    128 x 104: 12.8 us against 13.1 with 7, 256 x 500 18.6 / 21.7, 512 x 350 18.8 /
+//    19.1, but 256 x 700 20.1 / 19.1 and beyond the line 512 x 400 21.1 / 19.6;
+//    spectral E_x 256 x 500 20.6 / 21.1, 256 x 700 22.6 / 21.6, 512 x 400 21.4 / 22.1).
+//    Other FP32 runs of these sizes take it only with rows outside 64 to 1024, row
+//    counts outside 16 to 1024, or once tuned.
 //  - The odd-extension y solve up to 2^21 nodes: that solve and the step kernel
 //    (10; 512 x 416: 28.7 against 32.1 with 7, 1024 x 840: 60.1 / 64.3, 2048 x
 //    400: 57.2 / 59.3, and 62.5 with 4).
@@ -469,10 +473,12 @@ cudaError_t enqueue_base(ehd_run* r, int cur) {
 
 // Whether the run's steps are one node per thread (k_push): FP32-compute runs
 // of up to 2^19 nodes whose rows the warp transforms take, unless a launch shape
-// was asked for.  Against the march form, us per step: 256 x 205 10.5 / 13.7,
-// 512 x 416 16.2 / 19.6, 512 x 1000 (BF16) 27.2 / 30.0, 1024 x 300 20.3 / 23.2;
-// at 1024 x 840 both take 39, and beyond the populations leave L2, where the
-// march form's fewer bytes win.
+// was asked for.  Against the march form, us per step: 256 x 205 10.4 / 13.7,
+// 512 x 416 16.2 / 19.6, 512 x 1000 27.5 / 30.3 (BF16 26.8 / 29.8), 1024 x 512 25.6
+// / 32.3.  The line: with FP64 storage the two are equal there (62.9) and the
+// march form wins beyond (1024 x 600 75.0 / 65.8); with FP32 and 16 bits a little
+// is left beyond it (1024 x 600 28.2 / 29.4, BF16 27.1 / 28.4), and at 1024 x 700
+// the march form wins (35.4 / 33.3, BF16 32.8 / 31.7).
 bool push_form(const ehd_run* r) {
   return !r->tuned && !r->real_f64 && !r->pert && !r->ex_spectral && r->step_kernel == 0 && r->slab_shift == 0 &&
          r->Nx >= 64 && r->Nx <= 1024 && r->Ny >= 16 && r->Ny <= 1024 && (long long)r->Nx * r->Ny <= kPushNodes;
@@ -580,7 +586,7 @@ cudaError_t enqueue_step(ehd_run* r, int cur, long k) {
 
 // Whether the run steps on chip: small FP32-compute runs (64 to 256 columns,
 // up to 128 rows, as far as two copies of the populations fit the shared
-// memory of 16 CTAs), for which a step costs 4.3 us at 64 x 52 and 6.2 at
+// memory of 16 CTAs), for which a step costs 4.4 us at 64 x 52 and 6.3 at
 // 128 x 104 against 13.8 and 14.5 with a kernel per phase; beyond, one
 // cluster's 16 SMs would take longer than the whole GPU.  Looked at once, by
 // the run's first step (batch members never take it), and not under capture.

@@ -516,11 +516,13 @@ int step_flux_blocks(int Nx, bool real_f64);
 cudaError_t launch_march(const StepArgs& a, int storage, bool real_f64, cudaStream_t s);
 int march_strips(int Nx, int cols_per_lane);
 int march_warps_per_sm(int storage, bool real_f64, int cols_per_lane, int ring_depth);
-// kernel attributes and tables for runs of this kind (storage < 0: the batch's)
+// attributes of all march kernels, on the current device
 cudaError_t march_set_attributes();
-// Poisson solve from the charge plane: forward row FFTs and the wavenumber
-// systems on s; the FP64 mean mode (and the wall-flux totals) on `side`
-// between the fork and join events when side != nullptr.
+// Poisson solve from the charge plane (or, with a.g, from the populations):
+// forward row FFTs, wavenumber systems and inverse FFTs on s.  The mean mode and
+// the wall-flux totals are in the launch of the wavenumber systems (FP64) or of
+// the inverse FFTs (FP32 rows of 64 to 1024, up to 1024 rows); otherwise a kernel
+// of their own, on `side` between the fork and join events when side != nullptr.
 cudaError_t launch_poisson(const PoissonArgs& a, bool real_f64, cudaStream_t s, cudaStream_t side, cudaEvent_t fork,
                            cudaEvent_t join, const cudaEvent_t* marks = nullptr);
 // row transforms of the FP64 path (k_fft64.cu); the spectrum they keep is S / Nx
@@ -549,7 +551,7 @@ cudaError_t poisson_set_attributes();
 bool fftw_supported(int Nx);
 cudaError_t launch_rfft_warp(const PoissonArgs& a, cudaStream_t s);
 cudaError_t launch_irfft_warp(const PoissonArgs& a, cudaStream_t s);
-// the forward transform after k_push (rows of 64 to 512)
+// the forward transform after k_push (rows of 64 to 1024)
 cudaError_t launch_rfft_push(const PoissonArgs& a, cudaStream_t s);
 // the inverse transform and, beside it and the wavenumber solve, the mean mode
 bool irfft_mean_supported(int Nx, int Ny);

@@ -22,8 +22,9 @@
 //   inverse   a warp per row -> potential, its band's edge rows to both
 //             neighbours
 // Every value is formed as the multi-kernel step forms it (same chunking, same
-// order of sums, slab boundaries included), so the results are the same bit
-// for bit; FP64 wall fluxes are summed by spare warps of the two wall CTAs.
+// order of sums, slab boundaries included, by the functions of march_dev.cuh,
+// fft_dev.cuh and sweep_dev.cuh, whose rounding is stated), so the results are
+// the same bit for bit; FP64 wall fluxes are summed by spare warps of the two wall CTAs.
 //
 // Why 16 CTAs: the march needs the SMs (13 K nodes x 260 instructions), and
 // two copies of the populations (36 floats a node) must fit beside the rest;
